@@ -1560,17 +1560,39 @@ int route_batch(pim_instance* const* insts, const int* replicas, int count, int 
   return PIM_OK;
 }
 
-// fused 0-5, mid-N general path 6, mid-N diagonal-encoded 7
-constexpr int kGroups = 8, kMidGroup = 6, kMidDiagGroup = 7;
+// fused integer 0-3, fused real-valued 4-6 (n <= 64, 128, 256) and its fixed-point datapath 7,
+// mid-N general path 8, mid-N diagonal-encoded 9
+constexpr int kGroups = 10, kRealGroup = 4, kFixedGroup = 7, kMidGroup = 8, kMidDiagGroup = 9;
+constexpr int kRealCap[4] = {64, 128, 256, 128};  // largest n of groups 4-7
 
+// Replicas per CTA of a real-valued group.  A CTA's sweep takes about kRowsBase + rows (in
+// units of one replica's share of the work; the rest is the chain of MMA, barriers and
+// write-back that every CTA walks), so small tiles win while SMs are free and large ones
+// once the grid runs in several waves.
+int real_tile_rows(const std::vector<int>& replicas, int sms) {
+  constexpr int kRowsBase = 64;
+  int best = 128;
+  long long best_cost = LLONG_MAX;
+  for (int rows : {32, 64, 128}) {
+    long long units = 0;
+    for (int r : replicas) units += (r + rows - 1) / rows;
+    const long long cost = (units + sms - 1) / sms * (kRowsBase + rows);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = rows;
+    }
+  }
+  return best;
+}
 
 // Launch description of one batch: problem descriptors, the unit lists of each kernel group
-// (fused: npad 128 | 256 x diagonal-encoded | general bias | real-valued; persistent mid-N),
+// (fused: npad 128 | 256 x diagonal-encoded | general bias, real-valued; persistent mid-N),
 // the large-N instances, and the layout of the one device buffer that holds them.
 struct BatchPlan {
   std::vector<Problem> probs;
   std::vector<int> route;
   std::vector<WorkItem> work[kGroups];
+  int rows[kGroups];  // replicas per work item
   int maxR = 0, max_words = 0, stride_max = 4;
   size_t work_off[kGroups] = {};
   size_t ready_off[kGroups] = {};  // fused groups: chunked-queue counter and ready flags
@@ -1704,6 +1726,20 @@ int build_plan(pim_instance* const* insts, int count, const int* replicas, const
     }
   }
   for (auto& w : B.work) w.clear();
+  std::fill(std::begin(B.rows), std::end(B.rows), 128);
+  auto group_of = [&](int k) {
+    if (B.route[k] == kMid) return B.probs[k].dk > 0 ? kMidDiagGroup : kMidGroup;
+    if (!insts[k]->real) return (insts[k]->npad <= 128 ? 0 : 1) + (insts[k]->diag ? 0 : 2);
+    if (B.probs[k].fix_w > 0) return kFixedGroup;
+    return kRealGroup + (insts[k]->n <= 64 ? 0 : insts[k]->n <= 128 ? 1 : 2);
+  };
+  {
+    std::vector<int> reps[kGroups];
+    for (int k = 0; k < count && !ref; ++k)
+      if (B.route[k] == kFused && insts[k]->real) reps[group_of(k)].push_back(replicas[k]);
+    for (int g = kRealGroup; g <= kFixedGroup; ++g)
+      if (!reps[g].empty()) B.rows[g] = real_tile_rows(reps[g], device_sms());
+  }
   for (int k = 0; k < count && !ref; ++k) {
     if (B.route[k] == kBig) {
       BigPlan plan;
@@ -1715,10 +1751,8 @@ int build_plan(pim_instance* const* insts, int count, const int* replicas, const
                                                   sizeof(float) * 3 * rpad + 256);
       continue;
     }
-    const int g = B.route[k] == kMid ? (B.probs[k].dk > 0 ? kMidDiagGroup : kMidGroup)
-                                     : (insts[k]->npad <= 128 ? 0 : 1) +
-                                           (insts[k]->real ? 4 : (insts[k]->diag ? 0 : 2));
-    for (int rb = 0; rb < replicas[k]; rb += 128) B.work[g].push_back({k, rb});
+    const int g = group_of(k);
+    for (int rb = 0; rb < replicas[k]; rb += B.rows[g]) B.work[g].push_back({k, rb});
   }
   // persistent launch: largest units first so the last wave is short
   for (int g : {kMidGroup, kMidDiagGroup})
@@ -1729,7 +1763,7 @@ int build_plan(pim_instance* const* insts, int count, const int* replicas, const
   for (int g = 0; g < kGroups; ++g) {
     B.work_off[g] = off;
     off += B.work[g].size() * sizeof(WorkItem);
-    if (g < 4 && !B.work[g].empty()) {
+    if (g < kRealGroup && !B.work[g].empty()) {
       off = align256(off);
       B.ready_off[g] = off;
       off += (B.work[g].size() + 1) * sizeof(unsigned int);
@@ -1799,6 +1833,7 @@ int enqueue_plan(const BatchPlan& B, char* d_buf, char* big_scratch, pim_instanc
       L.probs = d_probs;
       L.work = reinterpret_cast<const WorkItem*>(d_buf + B.work_off[g]);
       L.nwork = static_cast<int>(B.work[g].size());
+      L.rows = B.rows[g];
       L.t_begin = t_begin;
       L.sweeps = sweeps;
       L.key_lo = static_cast<uint32_t>(seed);
@@ -1811,7 +1846,7 @@ int enqueue_plan(const BatchPlan& B, char* d_buf, char* big_scratch, pim_instanc
       L.inject = g_inject.load();
       L.next = reinterpret_cast<unsigned int*>(d_buf + B.counters_off);
       int blocks = L.nwork;
-      if (g < 4) {
+      if (g < kRealGroup) {
         // More units than the two CTAs per SM that run at once: cut every unit's sweeps into
         // chunks and let persistent CTAs take them from a queue, so that no SM idles or
         // runs a lone CTA while others finish a last partial wave (about kQueueDepth
@@ -1828,8 +1863,9 @@ int enqueue_plan(const BatchPlan& B, char* d_buf, char* big_scratch, pim_instanc
         const int blocks = std::min(L.nwork, sweep_mid_max_blocks());
         if (blocks < 1) return fail(PIM_ERR_CUDA, "anneal: mid-N kernel cannot be resident");
         CK(launch_sweep_mid(L, blocks, st, g == kMidDiagGroup), "persistent mid-N sweep kernel");
-      } else if (g >= 4) {
-        CK(launch_sweep_float(L, (g & 1) ? 256 : 128, L.nwork, st), "real-valued sweep kernel");
+      } else if (g >= kRealGroup) {
+        CK(launch_sweep_float(L, kRealCap[g - kRealGroup], g == kFixedGroup, L.nwork, st),
+           "real-valued sweep kernel");
       } else {
         CK(launch_sweep_tc(L, (g & 1) ? 256 : 128, blocks, st, g < 2), "fused sweep kernel");
       }

@@ -361,6 +361,7 @@ int pim_mimo_server::setup_device_queue() {
   Q.nslots = nslots;
   Q.idle_ns = static_cast<uint64_t>(cfg.idle_s * 1e9);
   L = pim::Launch{};
+  L.rows = cfg.replicas <= 32 ? 32 : cfg.replicas <= 64 ? 64 : 128;
   L.t_begin = 0;
   L.sweeps = cfg.sweeps;
   L.key_lo = static_cast<uint32_t>(cfg.seed);
@@ -399,7 +400,7 @@ int pim_mimo_server::ensure_kernel() {
     }
   }
   if (cudaMemsetAsync(d_exit, 0, 2 * sizeof(int), kstream) != cudaSuccess) return PIM_ERR_CUDA;
-  if (pim::launch_serve_float(L, Q, npad, ctas, kstream) != cudaSuccess) return PIM_ERR_CUDA;
+  if (pim::launch_serve_float(L, Q, n, ctas, kstream) != cudaSuccess) return PIM_ERR_CUDA;
   if (cudaEventRecord(kdone, kstream) != cudaSuccess) return PIM_ERR_CUDA;
   kernel_launched = true;
   return PIM_OK;

@@ -125,6 +125,18 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
       : "memory");
 }
 
+// True on one lane of a converged warp.  A warp that issues tcgen05.mma runs its whole loop
+// converged and lets this lane issue: the compiler then keeps descriptors and addresses in
+// uniform registers.  A loop run by one lane alone (if (lane == 0)) moves them there before
+// every MMA: 84 cycles per MMA on an otherwise idle SM, against 53 / 65 / 128 at N = 64 / 128 /
+// 256 this way, which is the tensor pipe's own pace (M = 128, FP8 and BF16).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(p));
+  return p != 0;
+}
+
 __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem),
                "r"(ncols)
@@ -275,12 +287,24 @@ __device__ __forceinline__ uint4 bf16x8_from_bits(uint32_t b) {
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
+// L-level staircase: level k = the largest with x >= its breakpoint -1 + 2 k / L (level 0 below
+// all of them).  (x + 1) L / 2 is within one of k up to 2^16 levels, so at most one breakpoint
+// on either side of it is compared; beyond that the breakpoints are searched.
 __device__ __forceinline__ float staircase(float x, int levels) {
   if (x < -1.0f) return -1.0f;
   if (x > 1.0f) return 1.0f;
+  auto breakpoint = [&](int k) { return -1.0f + 2.0f * k / levels; };
   int k = 0;
-  for (int kk = 1; kk < levels; ++kk)
-    if (x >= -1.0f + 2.0f * kk / levels) k = kk;
+  if (levels <= 65536) {
+    k = min(max(static_cast<int>((x + 1.0f) * 0.5f * levels), 0), levels - 1);
+    if (k > 0 && x < breakpoint(k))
+      --k;
+    else if (k + 1 < levels && x >= breakpoint(k + 1))
+      ++k;
+  } else {
+    for (int kk = 1; kk < levels; ++kk)
+      if (x >= breakpoint(kk)) k = kk;
+  }
   return -1.0f + 2.0f * k / (levels - 1);
 }
 
