@@ -317,10 +317,11 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_big_kernel(const __grid_con
   if (!grid_barrier(L.bar, bar_target, L.err, sFlag, L.wait_ns)) goto teardown;
 
   {
-    uint32_t loads = 0, mmas = 0, done_phase = 0;
+    // ring positions: stage and phase of the next load (the first round waits for nothing) / MMA
+    uint32_t ld_stage = 0, ld_phase = 0xFFFFFFFFu, mma_stage = 0, mma_phase = 0, done_phase = 0;
     const uint32_t idesc = REAL ? idesc_bf16(128, NT) : (FP4 ? idesc_mxf4(128, NT) : idesc_e4m3(128, NT));
     bool jres_ready = !FP4;
-    // Producer (thread 0): stream the K blocks of image `img` (spins of the tile) and, unless
+    // Producer (warp 0, converged, one elected lane): stream the K blocks of image `img` (spins of the tile) and, unless
     // they are resident, of the coupling rows of the column block into the ring.  A stage
     // is refilled once the MMAs that read it have completed (its empty barrier).
     // A stage holds kKPS consecutive K-blocks: the tile's spins of all of them in one copy
@@ -336,60 +337,79 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_big_kernel(const __grid_con
       for (int si = 0; si < nst; ++si) {
         const int kb0 = (rev ? nst - 1 - si : si) * kKPS;
         const int nk = kblocks - kb0 < kKPS ? kblocks - kb0 : kKPS;
-        const uint32_t s = loads % kStages, use = loads / kStages;
-        if (use > 0 && !mbar_wait_fast(bar_empty0 + 8 * s, (use - 1) & 1, L.wait_ns)) return false;
-        mbar_expect_tx(bar_full0 + 8 * s, nk * (kABytes + kBBytes));
-        bulk_g2s(smem_u32(sA + s * kKPS * kABytes), a_src + static_cast<size_t>(kb0) * kABytes,
-                 nk * kABytes, bar_full0 + 8 * s);
-        if constexpr (kBBytes > 0) {
-          if constexpr (NT == 128) {
-            bulk_g2s(smem_u32(sB + s * kKPS * kBBytes), b_src + static_cast<size_t>(kb0) * 16384,
-                     nk * kBBytes, bar_full0 + 8 * s);
-          } else {
-            for (int j = 0; j < nk; ++j)
-              bulk_g2s(smem_u32(sB + (s * kKPS + j) * kBBytes), b_src + static_cast<size_t>(kb0 + j) * 16384,
-                       kBBytes, bar_full0 + 8 * s);
+        const uint32_t s = ld_stage;
+        if (!__all_sync(0xFFFFFFFFu, ld_phase == 0xFFFFFFFFu ||
+                                         mbar_wait_fast(bar_empty0 + 8 * s, ld_phase & 1, L.wait_ns)))
+          return false;
+        if (elect_one()) {
+          mbar_expect_tx(bar_full0 + 8 * s, nk * (kABytes + kBBytes));
+          bulk_g2s(smem_u32(sA) + s * kKPS * kABytes, a_src + static_cast<size_t>(kb0) * kABytes,
+                   nk * kABytes, bar_full0 + 8 * s);
+          if constexpr (kBBytes > 0) {
+            if constexpr (NT == 128) {
+              bulk_g2s(smem_u32(sB) + s * kKPS * kBBytes, b_src + static_cast<size_t>(kb0) * 16384,
+                       nk * kBBytes, bar_full0 + 8 * s);
+            } else {
+#pragma unroll
+              for (int j = 0; j < kKPS; ++j)
+                if (j < nk)
+                  bulk_g2s(smem_u32(sB) + (s * kKPS + j) * kBBytes,
+                           b_src + static_cast<size_t>(kb0 + j) * 16384, kBBytes, bar_full0 + 8 * s);
+            }
           }
         }
-        ++loads;
+        __syncwarp();
+        if (++ld_stage == static_cast<uint32_t>(kStages)) {
+          ld_stage = 0;
+          ++ld_phase;
+        }
       }
       return true;
     };
-    // MMA issuer (thread 32): D = S_tile x J_block^T, K block by K block as stages land; it
-    // never waits for an MMA to finish, only for data.  Each MMA consumes 32 bytes of K
-    // (32 FP8, 16 BF16 or 64 E2M1 values).
+    // MMA issuer (warp 1, converged, one elected lane): D = S_tile x J_block^T, K block by K
+    // block as stages land; it never waits for an MMA to finish, only for data.  Each MMA
+    // consumes 32 bytes of K (32 FP8, 16 BF16 or 64 E2M1 values).
     auto multiply = [&](bool rev) -> bool {
       if (!jres_ready) {
-        if (!mbar_wait_fast(bar_jres, 0, L.wait_ns)) return false;
+        if (!__all_sync(0xFFFFFFFFu, mbar_wait_fast(bar_jres, 0, L.wait_ns))) return false;
         jres_ready = true;
       }
+      const uint64_t a_desc = sw128_desc(smem_u32(sA)), b_desc = sw128_desc(smem_u32(FP4 ? sJ : sB));
       const int nst = (kblocks + kKPS - 1) / kKPS;
       for (int si = 0; si < nst; ++si) {
         const int kb0 = (rev ? nst - 1 - si : si) * kKPS;
         const int nk = kblocks - kb0 < kKPS ? kblocks - kb0 : kKPS;
-        const uint32_t s = mmas % kStages, use = mmas / kStages;
-        if (!mbar_wait_fast(bar_full0 + 8 * s, use & 1, L.wait_ns)) return false;
+        const uint32_t s = mma_stage;
+        if (!__all_sync(0xFFFFFFFFu, mbar_wait_fast(bar_full0 + 8 * s, mma_phase & 1, L.wait_ns))) return false;
         tc_fence_after();
-        for (int j = 0; j < nk; ++j) {
-          const uint32_t a0 = smem_u32(sA + (s * kKPS + j) * kABytes);
-          const uint32_t b0 = FP4 ? smem_u32(sJ + (kb0 + j) * NT * 128)
-                                  : smem_u32(sB + (s * kKPS + j) * kBBytes);
+        if (elect_one()) {
+          const uint64_t a0 = a_desc + s * (kKPS * kABytes >> 4);
+          const uint64_t b0 = b_desc + (FP4 ? kb0 * (NT * 128 >> 4) : s * (kKPS * kBBytes >> 4));
 #pragma unroll
-          for (int ks = 0; ks < 4; ++ks) {
-            const uint32_t acc = (si > 0 || j > 0 || ks > 0) ? 1u : 0u;
-            if constexpr (REAL)
-              mma_bf16(tmem, sw128_desc(a0 + ks * 32), sw128_desc(b0 + ks * 32), idesc, acc);
-            else if constexpr (FP4)
-              mma_mxf4(tmem, sw128_desc(a0 + ks * 32), sw128_desc(b0 + ks * 32), idesc, tmem + NT,
-                       tmem + NT, acc);
-            else
-              mma_e4m3(tmem, sw128_desc(a0 + ks * 32), sw128_desc(b0 + ks * 32), idesc, acc);
-          }
+          for (int j = 0; j < kKPS; ++j)
+            if (j < nk) {
+#pragma unroll
+              for (int ks = 0; ks < 4; ++ks) {
+                const uint32_t acc = (si > 0 || j > 0 || ks > 0) ? 1u : 0u;
+                const uint64_t a = a0 + j * (kABytes >> 4) + 2 * ks;
+                const uint64_t b = b0 + j * ((FP4 ? NT * 128 : kBBytes) >> 4) + 2 * ks;
+                if constexpr (REAL)
+                  mma_bf16(tmem, a, b, idesc, acc);
+                else if constexpr (FP4)
+                  mma_mxf4(tmem, a, b, idesc, tmem + NT, tmem + NT, acc);
+                else
+                  mma_e4m3(tmem, a, b, idesc, acc);
+              }
+            }
+          mma_commit(bar_empty0 + 8 * s);
+          if (si + 1 == nst) mma_commit(bar_done);
         }
-        mma_commit(bar_empty0 + 8 * s);
-        ++mmas;
+        __syncwarp();
+        if (++mma_stage == static_cast<uint32_t>(kStages)) {
+          mma_stage = 0;
+          ++mma_phase;
+        }
       }
-      mma_commit(bar_done);
       return true;
     };
 
@@ -421,16 +441,16 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_big_kernel(const __grid_con
     uint32_t prev = 0;  // s(t-1) of this thread's spins, until its energy has been tracked
     for (int t = t_begin; t <= t_end; ++t) {
       const bool last = t == t_end;
-      if (tid == 0) {
+      if (warp == 0) {
         fence_proxy_async_global();
         // Injected fault: nothing is loaded in the first sweep, so the MMA thread's first
         // wait cannot complete.
-        if (!(L.inject == 1 && t == t_begin) && !produce(L.s_img[cur_img], kRev && (t & 1))) {
+        if (!(L.inject == 1 && t == t_begin) && !produce(L.s_img[cur_img], kRev && (t & 1)) && lane == 0) {
           atomicOr(L.err, kDevErrTimeout);
           grid_abort(L.bar);
         }
-      } else if (tid == 32) {
-        if (!multiply(kRev && (t & 1))) {
+      } else if (warp == 1) {
+        if (!multiply(kRev && (t & 1)) && lane == 0) {
           atomicOr(L.err, kDevErrTimeout);
           grid_abort(L.bar);
         }
