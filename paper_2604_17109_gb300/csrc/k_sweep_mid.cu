@@ -293,8 +293,8 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
     const int nchunks = npad / kNT, kblocks = npad / 128;
     const int t_begin = L.t_begin, t_end = L.t_begin + L.sweeps;
 
-    if (tid == 0) {
-      // ---- producer: coupling K-blocks (chunk-major) into the ring ---------------------
+    if (warp == 0) {
+      // ---- producer (converged warp, one elected lane): coupling K-blocks into the ring ---
       bool ok = true;
       for (int t = t_begin; t <= t_end && ok; ++t) {
         if (L.inject == 1 && first_unit && t == t_begin) continue;  // injected fault
@@ -302,37 +302,42 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
           for (int kb0 = 0; kb0 < kblocks; kb0 += kKPS) {
             const int nk = kblocks - kb0 < kKPS ? kblocks - kb0 : kKPS;
             const uint32_t s = loads % kStages, use = loads / kStages;
-            if ((use > 0 && !wait_phase(empty0 + 8 * s, (use - 1) & 1, L.wait_ns)) ||
-                *sAbort != 0) {
+            if (!__all_sync(0xFFFFFFFFu, (use == 0 || wait_phase(empty0 + 8 * s, (use - 1) & 1, L.wait_ns)) &&
+                                             *sAbort == 0)) {
               ok = false;
               break;
             }
-            mbar_expect_tx(full0 + 8 * s, nk * kBlockBytes);
-            if (npad > 256) {
-              // images of n > 256 (npad >= 512) are chunk-major: the stage's K-blocks of chunk
-              // c are contiguous, one copy
-              bulk_g2s(smem_u32(sRing + s * kStageBytes),
-                       P.jimg + (static_cast<size_t>(c) * kblocks + kb0) * kBlockBytes, nk * kBlockBytes,
-                       full0 + 8 * s);
-            } else {
-              for (int j = 0; j < nk; ++j)
-                bulk_g2s(smem_u32(sRing + s * kStageBytes + j * kBlockBytes),
-                         P.jimg + static_cast<size_t>(kb0 + j) * npad * 128 + static_cast<size_t>(c) * kNT * 128,
-                         kBlockBytes, full0 + 8 * s);
+            if (elect_one()) {
+              mbar_expect_tx(full0 + 8 * s, nk * kBlockBytes);
+              if (npad > 256) {
+                // images of n > 256 (npad >= 512) are chunk-major: the stage's K-blocks of chunk
+                // c are contiguous, one copy
+                bulk_g2s(smem_u32(sRing) + s * kStageBytes,
+                         P.jimg + (static_cast<size_t>(c) * kblocks + kb0) * kBlockBytes, nk * kBlockBytes,
+                         full0 + 8 * s);
+              } else {
+                for (int j = 0; j < nk; ++j)
+                  bulk_g2s(smem_u32(sRing) + s * kStageBytes + j * kBlockBytes,
+                           P.jimg + static_cast<size_t>(kb0 + j) * npad * 128 + static_cast<size_t>(c) * kNT * 128,
+                           kBlockBytes, full0 + 8 * s);
+              }
             }
+            __syncwarp();
             ++loads;
           }
       }
-      if (!ok) {
+      if (!ok && lane == 0) {
         atomicOr(L.err, kDevErrTimeout);
         *sAbort = 1;
       }
-    } else if (tid == 32) {
-      // ---- MMA issuer: per sweep, wait for s(t) in the A image, then every chunk --------
+    } else if (warp == 1) {
+      // ---- MMA issuer (converged warp, one elected lane): per sweep, wait for s(t) in the A
+      // image, then every chunk --------------------------------------------------------------
       const uint32_t idesc_u = P.e5m2 ? idesc_e5m2(128, kNT) : idesc;
+      const uint64_t ring_desc = sw128_desc(smem_u32(sRing));
       bool ok = true;
       for (int t = t_begin; t <= t_end && ok; ++t) {
-        if (!wait_phase(aready, apass & 1, L.wait_ns)) {
+        if (!__all_sync(0xFFFFFFFFu, wait_phase(aready, apass & 1, L.wait_ns))) {
           ok = false;
           break;
         }
@@ -340,7 +345,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
         tc_fence_after();
         for (int c = 0; c < nchunks && ok; ++c) {
           const uint32_t b = cpass % kBufs, buse = cpass / kBufs;
-          if (buse > 0 && !wait_phase(tempty0 + 8 * b, (buse - 1) & 1, L.wait_ns)) {
+          if (!__all_sync(0xFFFFFFFFu, buse == 0 || wait_phase(tempty0 + 8 * b, (buse - 1) & 1, L.wait_ns))) {
             ok = false;
             break;
           }
@@ -348,28 +353,33 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
           for (int kb0 = 0; kb0 < kblocks; kb0 += kKPS) {
             const int nk = kblocks - kb0 < kKPS ? kblocks - kb0 : kKPS;
             const uint32_t s = mmas % kStages, use = mmas / kStages;
-            if (!wait_phase(full0 + 8 * s, use & 1, L.wait_ns)) {
+            if (!__all_sync(0xFFFFFFFFu, wait_phase(full0 + 8 * s, use & 1, L.wait_ns))) {
               ok = false;
               break;
             }
             tc_fence_after();
-            for (int j = 0; j < nk; ++j) {
-              const int kb = kb0 + j;
-              const uint32_t b0 = smem_u32(sRing + s * kStageBytes + j * kBlockBytes);
+            if (elect_one()) {
+              const uint64_t b0 = ring_desc + s * (kStageBytes >> 4);
+              const uint32_t a0 = tmem + kTmemA + kb0 * 32, d = tmem + b * kNT;
 #pragma unroll
-              for (int ks = 0; ks < 4; ++ks)
-                mma_f8_ta(tmem + b * kNT, tmem + kTmemA + kb * 32 + ks * 8, sw128_desc(b0 + ks * 32),
-                          idesc_u, (kb > 0 || ks > 0) ? 1u : 0u);
+              for (int j = 0; j < kKPS; ++j)
+                if (j < nk) {
+#pragma unroll
+                  for (int ks = 0; ks < 4; ++ks)
+                    mma_f8_ta(d, a0 + j * 32 + ks * 8, b0 + j * (kBlockBytes >> 4) + 2 * ks, idesc_u,
+                              (kb0 > 0 || j > 0 || ks > 0) ? 1u : 0u);
+                }
+              mma_commit(empty0 + 8 * s);
+              if (kb0 + kKPS >= kblocks) mma_commit(tfull0 + 8 * b);
             }
-            mma_commit(empty0 + 8 * s);
+            __syncwarp();
             ++mmas;
           }
           if (!ok) break;
-          mma_commit(tfull0 + 8 * b);
           ++cpass;
         }
       }
-      if (!ok) {
+      if (!ok && lane == 0) {
         atomicOr(L.err, kDevErrTimeout);
         *sAbort = 1;
       }

@@ -295,20 +295,26 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_tc_kernel(const Launch L) {
     __syncthreads();
 
     const uint32_t idesc = idesc_e4m3(kTileM, mma_n);
-    const uint32_t sA_addr = smem_u32(sA), sJ_addr = smem_u32(sJ);
+    // Warp 0, converged: the elected lane issues the fields' MMAs.
+    const uint64_t a_desc = sw128_desc(smem_u32(sA)), j_desc = sw128_desc(smem_u32(sJ));
     auto issue_fields = [&]() {
-      for (int ks = 0; ks < ksteps; ++ks) {
-        const uint32_t kb = ks >> 2, ko = (ks & 3) * 32;
-        mma_e4m3(tmem, sw128_desc(sA_addr + kb * (kTileM * 128) + ko),
-                 sw128_desc(sJ_addr + kb * (NPAD * 128) + ko), idesc, ks > 0 ? 1u : 0u);
+      if (elect_one()) {
+#pragma unroll
+        for (int ks = 0; ks < NPAD / 32; ++ks)
+          if (ks < ksteps)
+            mma_e4m3(tmem, a_desc + (ks >> 2) * (kTileM * 128 >> 4) + 2 * (ks & 3),
+                     j_desc + (ks >> 2) * (NPAD * 128 >> 4) + 2 * (ks & 3), idesc, ks > 0 ? 1u : 0u);
+        mma_commit(bar_mma);
       }
-      mma_commit(bar_mma);
+      __syncwarp();
     };
 
-    if (tid == 0) {
-      if (!mbar_wait_bounded(bar_j, jphase, L.wait_ns)) {
-        atomicOr(L.err, kDevErrTimeout);
-        *sAbort = 1;
+    if (warp == 0) {
+      if (!__all_sync(0xFFFFFFFFu, mbar_wait_bounded(bar_j, jphase, L.wait_ns))) {
+        if (lane == 0) {
+          atomicOr(L.err, kDevErrTimeout);
+          *sAbort = 1;
+        }
       } else if (L.inject != 1) {  // injected fault: the first wait below cannot complete
         tc_fence_after();
         issue_fields();
@@ -410,7 +416,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_tc_kernel(const Launch L) {
       __syncthreads();
       aborted = *sAbort != 0;
       if (aborted) break;
-      if (tid == 0) {
+      if (warp == 0) {
         tc_fence_after();
         issue_fields();  // fields of s(t+1)
       }
