@@ -244,6 +244,49 @@ cudaError_t launch_gather_copy(const CopyJob* d_jobs, int count, cudaStream_t st
   return cudaGetLastError();
 }
 
+// ---------------------------------------------------------------------------------------
+// Record copy: every record of one instance in one launch, one grid row per record.  The copies
+// are small (hundreds of bytes to a few hundred KB), so what they cost is their commands:
+// measured on a stream with 152 instances x 256 replicas, n = 512, four records took 15.0 us an
+// instance as copy calls (3.7 each), 1.7 us as this launch (4.1 with ordinary stream order).
+// 16 bytes per thread and step where both sides are aligned, else 4.
+// ---------------------------------------------------------------------------------------
+__global__ void record_copy_kernel(const __grid_constant__ RecordCopy rc) {
+  const unsigned long long t0 = static_cast<unsigned long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+  const unsigned long long step = static_cast<unsigned long long>(gridDim.x) * blockDim.x;
+  // the next copy of the stream may be set up now; this one's data is there once every earlier
+  // kernel has ended
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const uint32_t* src = rc.src[blockIdx.y];
+  uint32_t* dst = rc.dst[blockIdx.y];
+  const unsigned long long words = rc.words[blockIdx.y];
+  unsigned long long done = 0;
+  if (((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0) {
+    for (unsigned long long i = t0; i < words / 4; i += step)
+      reinterpret_cast<uint4*>(dst)[i] = reinterpret_cast<const uint4*>(src)[i];
+    done = words & ~3ull;
+  }
+  for (unsigned long long i = done + t0; i < words; i += step) dst[i] = src[i];
+}
+
+cudaError_t launch_record_copy(const RecordCopy& rc, cudaStream_t st) {
+  unsigned long long most = 0;
+  for (int k = 0; k < rc.count; ++k) most = rc.words[k] > most ? rc.words[k] : most;
+  if (most == 0) return cudaSuccess;
+  const unsigned long long want = (most + 1023) / 1024;  // 256 threads x 16 bytes
+  cudaLaunchAttribute early{};
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>(want < 152 ? want : 152), rc.count);
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cfg.attrs = &early;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, record_copy_kernel, rc);
+}
+
 // One word from device memory into mapped pinned host memory (the error-word mirror).
 __global__ void mirror_word_kernel(const int* __restrict__ d, int* h) {
   *reinterpret_cast<volatile int*>(h) = *reinterpret_cast<const volatile int*>(d);

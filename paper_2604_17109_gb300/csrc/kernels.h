@@ -49,6 +49,9 @@ cudaError_t launch_mirror_word(const int* d, int* h_dev, cudaStream_t st);
 // Copies every job's block (jobs in device memory).
 cudaError_t launch_gather_copy(const CopyJob* d_jobs, int count, cudaStream_t st);
 
+// Copies one instance's records device to device (nothing when there are none).
+cudaError_t launch_record_copy(const RecordCopy& rc, cudaStream_t st);
+
 // Initial spin bits: from Philox (d_init == nullptr) or from int8 +-1 spins [R][n].
 cudaError_t launch_init_bits(const Problem* d_probs, int nprob, int maxR, int max_words,
                              const int8_t* d_init, uint32_t key_lo, uint32_t key_hi,

@@ -74,6 +74,23 @@ struct CopyJob {
   unsigned long long bytes;
 };
 
+// The records of one instance that one launch copies device to device (4-byte words).
+struct RecordCopy {
+  const uint32_t* src[6];
+  uint32_t* dst[6];
+  unsigned long long words[6];
+  int count;
+
+  // Adds a copy of `bytes` (a multiple of 4, 4-byte aligned on both sides) unless `fits` is false.
+  bool add(void* d, const void* s, size_t bytes, bool fits) {
+    if (!fits || reinterpret_cast<uintptr_t>(d) % 4 != 0) return false;
+    src[count] = static_cast<const uint32_t*>(s);
+    dst[count] = static_cast<uint32_t*>(d);
+    words[count++] = bytes / 4;
+    return true;
+  }
+};
+
 // One unit of work of the fused sweep kernel: (problem index, first replica).
 struct WorkItem {
   int prob;

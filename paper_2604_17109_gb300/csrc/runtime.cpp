@@ -235,6 +235,7 @@ cudaError_t upload_async(void* dst, const void* src, size_t bytes, cudaStream_t 
 struct RunEvent {
   cudaEvent_t ev = nullptr;
   int device = 0;
+  unsigned long long stream_id = 0;  // of the stream it was recorded on (never reused); 0 unknown
   ~RunEvent() { give_event(device, ev); }
 };
 
@@ -1954,6 +1955,10 @@ int finish_run(pim_instance* const* insts, int count, const int* replicas,
   done->device = insts[0]->device;
   CK(take_event(done->device, &done->ev), "cudaEventCreate");
   CK(cudaEventRecord(done->ev, st), "cudaEventRecord");
+  if (cudaStreamGetId(st, &done->stream_id) != cudaSuccess) {
+    cudaGetLastError();
+    done->stream_id = 0;
+  }
   for (int k = 0; k < count; ++k) {
     insts[k]->h_res_valid = to_host;
     insts[k]->R = replicas[k];
@@ -2564,23 +2569,80 @@ int copy_state(pim_instance* inst, const uint32_t* d_bits, int8_t* out) {
 }
 }  // namespace
 
+namespace {
+
+// Whether work enqueued on st now follows the run by stream order alone (a wait between two
+// commands of one stream costs about 2 us of it).  Streams are told apart by their id, which,
+// unlike a handle, no later stream takes over; a capture in progress starts a new order.
+bool follows_in_stream(const RunEvent& run, cudaStream_t st) {
+  unsigned long long id = 0;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusActive;
+  if (run.stream_id == 0 || cudaStreamGetId(st, &id) != cudaSuccess ||
+      cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return id == run.stream_id && cs == cudaStreamCaptureStatusNone;
+}
+
+// Whether dst .. dst + bytes lies inside one allocation of plain device memory of `device`.
+bool writable_device_range(const void* dst, size_t bytes, int device) {
+  using RangeFn = int (*)(unsigned long long*, size_t*, unsigned long long);
+  static const RangeFn range = [] {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 12000, cudaEnableDefault, &found) !=
+            cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      fn = nullptr;
+    }
+    return reinterpret_cast<RangeFn>(fn);
+  }();
+  cudaPointerAttributes at{};
+  if (!range || cudaPointerGetAttributes(&at, dst) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (at.type != cudaMemoryTypeDevice || at.device != device) return false;
+  unsigned long long base = 0;
+  size_t size = 0;
+  const unsigned long long p = reinterpret_cast<unsigned long long>(dst);
+  return range(&base, &size, p) == 0 && p >= base && bytes <= base + size - p;
+}
+
+}  // namespace
+
 PIM_API int pim_results_dev(pim_instance* inst, double* best_E, int32_t* best_t,
                             int32_t* first_hit_t, double* final_E, uint32_t* best_bits,
                             uint32_t* final_bits, void* cuda_stream) {
   if (!inst) return fail(PIM_ERR_INVALID, "pim_results_dev: instance is NULL");
   if (!inst->has_results) return fail(PIM_ERR_STATE, "pim_results_dev: no anneal has run");
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  if (inst->done) CK(cudaStreamWaitEvent(st, inst->done->ev, 0), "cudaStreamWaitEvent");
+  if (inst->done && !follows_in_stream(*inst->done, st))
+    CK(cudaStreamWaitEvent(st, inst->done->ev, 0), "cudaStreamWaitEvent");
   const size_t R = inst->R, bits = R * inst->words * sizeof(uint32_t);
-  auto d2d = [&](void* dst, const void* src, size_t bytes) {
-    return dst ? cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToDevice, st) : cudaSuccess;
+  struct Record {
+    void* dst;
+    const void* src;
+    size_t bytes;
+    const char* what;
   };
-  CK(d2d(best_E, inst->d_bestE, R * 8), "copy best energies");
-  CK(d2d(final_E, inst->d_finalE, R * 8), "copy final energies");
-  CK(d2d(best_t, inst->d_bestT, R * 4), "copy best steps");
-  CK(d2d(first_hit_t, inst->d_first, R * 4), "copy first hits");
-  CK(d2d(best_bits, inst->d_best_bits, bits), "copy best states");
-  CK(d2d(final_bits, inst->d_cur_bits, bits), "copy final states");
+  const Record recs[6] = {{best_E, inst->d_bestE, R * 8, "copy best energies"},
+                          {final_E, inst->d_finalE, R * 8, "copy final energies"},
+                          {best_t, inst->d_bestT, R * 4, "copy best steps"},
+                          {first_hit_t, inst->d_first, R * 4, "copy first hits"},
+                          {best_bits, inst->d_best_bits, bits, "copy best states"},
+                          {final_bits, inst->d_cur_bits, bits, "copy final states"}};
+  // One launch for every record that lies in this device's memory; others (and one that does
+  // not fit its allocation) go to the copy call, which checks them.
+  RecordCopy rc{};
+  for (const Record& r : recs) {
+    if (!r.dst) continue;
+    if (rc.add(r.dst, r.src, r.bytes, writable_device_range(r.dst, r.bytes, inst->device))) continue;
+    CK(cudaMemcpyAsync(r.dst, r.src, r.bytes, cudaMemcpyDeviceToDevice, st), r.what);
+  }
+  CK(launch_record_copy(rc, st), "copy records");
   return PIM_OK;
 }
 
