@@ -191,7 +191,8 @@ __global__ void __launch_bounds__(FloatCfg<CAP>::kBoundThreads, 1)
   const bool decides = warp < NW, sums = warp >= NW && warp < NW + ewarps;
   const bool multiplies = warp == NW + ewarps;
   // decision warps: (warp / 4, copy of the replica group) is the slot; chunks slot + j NW / nrg
-  const int slot = (warp >> 2) * (4 / nrg) + quad / nrg;
+  const int lg = nrg >> 1;           // log2(nrg)
+  const int step = NW >> lg, slot = (warp >> 2) * (4 >> lg) + (quad >> lg);
   const uint32_t bar_mma0 = smem_u32(&bars[0]);  // [2]: fields in accumulator 0 / 1
   const uint32_t bar_ready = smem_u32(&bars[2]);  // spins written by every decision warp
   const uint32_t bar_sum0 = smem_u32(&bars[3]);   // [2]: energy of state m & 1 summed
@@ -288,7 +289,7 @@ __global__ void __launch_bounds__(FloatCfg<CAP>::kBoundThreads, 1)
       float* const fields = SERVE ? nullptr : P.fields_out;
       const int nchw = nch * (16 / W);
       uint8_t* bits8 = reinterpret_cast<uint8_t*>(sBits);
-      const int copies = 4 / nrg, copy_bytes = 4096 * nrg;
+      const int copies = 4 >> lg, copy_bytes = 4096 * nrg;
       // spins c W .. c W + W - 1 of this thread's replica in state buffer b
       auto bits_at = [&](uint32_t b, int c) {
         return bits8 + ((b * G + c * W / 16) * kTileM + rep) * 2 + (W == 8 ? (c & 1) : 0);
@@ -314,7 +315,7 @@ __global__ void __launch_bounds__(FloatCfg<CAP>::kBoundThreads, 1)
       };
       // s(t_begin)
       if (grp_active)
-        for (int c = slot; c < nchw; c += NW / nrg) {
+        for (int c = slot; c < nchw; c += step) {
           uint32_t nb = 0;
           if (row_valid) {
             if constexpr (SERVE) {
@@ -369,7 +370,7 @@ __global__ void __launch_bounds__(FloatCfg<CAP>::kBoundThreads, 1)
         };
         if (grp_active)
 #pragma unroll 1
-          for (int c = slot; c < nchw; c += NW / nrg) {
+          for (int c = slot; c < nchw; c += step) {
             const uint32_t ob = W == 16 ? *reinterpret_cast<const uint16_t*>(bits_at(m & 1, c)) : *bits_at(m & 1, c);
             uint32_t rw[W / 2];
 #pragma unroll

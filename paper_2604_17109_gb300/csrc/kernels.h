@@ -63,6 +63,11 @@ cudaError_t launch_sweep_tc(const Launch& L, int npad_max, int blocks, cudaStrea
                             bool diag);
 int sweep_tc_smem_bytes(int npad, int stride_words_max);
 
+// The same sweeps with the shortest chain per sweep, for launches of few tiles: one CTA per work
+// item of L.rows (32, 64 or 128) replicas, every n <= nmax <= 256.
+cudaError_t launch_sweep_lat(const Launch& L, int nmax, int blocks, cudaStream_t st, bool diag);
+bool sweep_lat_fits(int stride_words_max);
+
 // Real-valued couplings (BF16 operands, FP32 decision), every n <= nmax <= 256, one CTA per
 // work item of L.rows (32, 64 or 128) replicas; fixed: the fixed-point datapath, nmax <= 128.
 cudaError_t launch_sweep_float(const Launch& L, int nmax, bool fixed, int blocks, cudaStream_t st);

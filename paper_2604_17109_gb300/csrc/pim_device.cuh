@@ -113,7 +113,7 @@ struct Launch {
   const Problem* probs;
   const WorkItem* work;
   int nwork;
-  int rows;                // real-valued kernel: replicas per work item (32, 64 or 128)
+  int rows;                // latency and real-valued kernels: replicas per work item (32, 64, 128)
   int t_begin;
   int sweeps;
   uint32_t key_lo, key_hi;

@@ -1566,24 +1566,57 @@ int route_batch(pim_instance* const* insts, const int* replicas, int count, int 
 constexpr int kGroups = 10, kRealGroup = 4, kFixedGroup = 7, kMidGroup = 8, kMidDiagGroup = 9;
 constexpr int kRealCap[4] = {64, 128, 256, 128};  // largest n of groups 4-7
 
-// Replicas per CTA of a real-valued group.  A CTA's sweep takes about kRowsBase + rows (in
-// units of one replica's share of the work; the rest is the chain of MMA, barriers and
-// write-back that every CTA walks), so small tiles win while SMs are free and large ones
-// once the grid runs in several waves.
-int real_tile_rows(const std::vector<int>& replicas, int sms) {
-  constexpr int kRowsBase = 64;
-  int best = 128;
-  long long best_cost = LLONG_MAX;
-  for (int rows : {32, 64, 128}) {
+// Tile heights of the kernels that replicate small tiles over the lane quadrants (k_sweep_lat.cu
+// and k_sweep_float.cu).  Measured us per sweep (GB300, n = 64, 128, 256) of a lone CTA and, per
+// CTA, of an SM with several: a launch takes about max(alone, CTAs per SM x full).  A smaller tile
+// shortens the sweep, a taller one does more per CTA, so small tiles win while SMs are free.
+constexpr int kTileRows[3] = {32, 64, 128};
+struct TileCost {
+  double alone[3], full[3];
+};
+constexpr TileCost kRealCost[3] = {{{1.00, 1.48, 2.57}, {0.73, 1.15, 2.57}},
+                                   {{1.76, 2.70, 4.01}, {1.74, 2.68, 4.01}},
+                                   {{3.40, 5.15, 8.60}, {3.38, 5.13, 8.60}}};
+constexpr TileCost kLatCost[2][3] = {{{{0.87, 1.25, 2.05}, {0.54, 0.82, 1.39}},   // diagonal-encoded
+                                      {{1.14, 1.58, 2.58}, {1.11, 1.57, 2.58}},
+                                      {{1.73, 2.54, 4.37}, {1.71, 2.54, 4.37}}},
+                                     {{{0.86, 1.24, 2.03}, {0.56, 1.23, 2.03}},   // general bias
+                                      {{1.25, 1.88, 3.20}, {1.24, 1.89, 3.20}},
+                                      {{2.03, 3.10, 5.62}, {2.01, 3.16, 5.66}}}};
+// The throughput kernel (k_sweep_tc.cu): a lone 128-replica tile, and per tile of a full SM.  Its
+// queue evens out partial waves.
+constexpr double kTcAlone[2][3] = {{1.20, 1.93, 4.28}, {1.94, 3.48, 7.25}};
+constexpr double kTcFull[2][3] = {{0.91, 1.59, 3.20}, {1.61, 3.01, 6.18}};
+
+int size_class(int n) { return n <= 64 ? 0 : n <= 128 ? 1 : 2; }
+
+// Tile height for `replicas` (one entry per instance) and its cost.
+int tile_rows(const std::vector<int>& replicas, const TileCost& c, int sms, double* cost) {
+  int best = 0;
+  *cost = 0.0;
+  for (int k = 0; k < 3; ++k) {
     long long units = 0;
-    for (int r : replicas) units += (r + rows - 1) / rows;
-    const long long cost = (units + sms - 1) / sms * (kRowsBase + rows);
-    if (cost < best_cost) {
-      best_cost = cost;
-      best = rows;
+    for (int r : replicas) units += (r + kTileRows[k] - 1) / kTileRows[k];
+    const double us = std::max(c.alone[k], static_cast<double>((units + sms - 1) / sms) * c.full[k]);
+    if (best == 0 || us < *cost) {
+      best = kTileRows[k];
+      *cost = us;
     }
   }
   return best;
+}
+
+// Replicas per CTA of an integer fused group when it runs on the latency kernel, or 0 where the
+// throughput kernel takes less (its tiles cover the SMs; the lines lie where the costs above
+// cross, e.g. n = 256: up to about 150 replica tiles of 32 or 64, with a bias any number).
+int lat_tile_rows(const std::vector<int>& replicas, int nmax, bool diag, int sms) {
+  const int k = size_class(nmax), d = diag ? 0 : 1;
+  long long tiles = 0;
+  for (int r : replicas) tiles += (r + 127) / 128;
+  const double tc_us = std::max(kTcAlone[d][k], kTcFull[d][k] * static_cast<double>(tiles) / sms);
+  double us = 0.0;
+  const int rows = tile_rows(replicas, kLatCost[d][k], sms, &us);
+  return us < tc_us ? rows : 0;
 }
 
 // Launch description of one batch: problem descriptors, the unit lists of each kernel group
@@ -1594,6 +1627,8 @@ struct BatchPlan {
   std::vector<int> route;
   std::vector<WorkItem> work[kGroups];
   int rows[kGroups];  // replicas per work item
+  int nmax[kGroups] = {};       // largest n of a group
+  bool lat[kGroups] = {};       // integer fused groups: latency kernel
   int maxR = 0, max_words = 0, stride_max = 4;
   size_t work_off[kGroups] = {};
   size_t ready_off[kGroups] = {};  // fused groups: chunked-queue counter and ready flags
@@ -1736,10 +1771,23 @@ int build_plan(pim_instance* const* insts, int count, const int* replicas, const
   };
   {
     std::vector<int> reps[kGroups];
-    for (int k = 0; k < count && !ref; ++k)
-      if (B.route[k] == kFused && insts[k]->real) reps[group_of(k)].push_back(replicas[k]);
-    for (int g = kRealGroup; g <= kFixedGroup; ++g)
-      if (!reps[g].empty()) B.rows[g] = real_tile_rows(reps[g], device_sms());
+    for (int k = 0; k < count && !ref; ++k) {
+      if (B.route[k] != kFused) continue;
+      const int g = group_of(k);
+      reps[g].push_back(replicas[k]);
+      B.nmax[g] = std::max(B.nmax[g], insts[k]->n);
+    }
+    for (int g = 0; g <= kFixedGroup; ++g) {
+      if (reps[g].empty()) continue;
+      if (g >= kRealGroup) {
+        double us = 0.0;
+        B.rows[g] = tile_rows(reps[g], kRealCost[size_class(kRealCap[g - kRealGroup])], device_sms(), &us);
+      } else if (sweep_lat_fits(B.stride_max)) {
+        const int rows = lat_tile_rows(reps[g], B.nmax[g], g < 2, device_sms());
+        B.lat[g] = rows > 0;
+        if (rows > 0) B.rows[g] = rows;
+      }
+    }
   }
   for (int k = 0; k < count && !ref; ++k) {
     if (B.route[k] == kBig) {
@@ -1847,7 +1895,7 @@ int enqueue_plan(const BatchPlan& B, char* d_buf, char* big_scratch, pim_instanc
       L.inject = g_inject.load();
       L.next = reinterpret_cast<unsigned int*>(d_buf + B.counters_off);
       int blocks = L.nwork;
-      if (g < kRealGroup) {
+      if (g < kRealGroup && !B.lat[g]) {
         // More units than the two CTAs per SM that run at once: cut every unit's sweeps into
         // chunks and let persistent CTAs take them from a queue, so that no SM idles or
         // runs a lone CTA while others finish a last partial wave (about kQueueDepth
@@ -1867,6 +1915,8 @@ int enqueue_plan(const BatchPlan& B, char* d_buf, char* big_scratch, pim_instanc
       } else if (g >= kRealGroup) {
         CK(launch_sweep_float(L, kRealCap[g - kRealGroup], g == kFixedGroup, L.nwork, st),
            "real-valued sweep kernel");
+      } else if (B.lat[g]) {
+        CK(launch_sweep_lat(L, B.nmax[g], L.nwork, st, g < 2), "fused sweep kernel (latency)");
       } else {
         CK(launch_sweep_tc(L, (g & 1) ? 256 : 128, blocks, st, g < 2), "fused sweep kernel");
       }

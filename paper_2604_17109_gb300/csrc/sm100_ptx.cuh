@@ -62,10 +62,12 @@ __device__ __forceinline__ void st_release_gpu(unsigned int* p, uint32_t v) {
 }
 
 // Wait for the phase with the given parity; gives up after `limit_ns` (0 = 2 s) and
-// returns false.
+// returns false.  The clock is read only once a number of polls have failed: reading it costs
+// more than the wait itself where a phase is a few hundred nanoseconds away.
 static __device__ __noinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
                                                       uint64_t limit_ns = 0) {
-  if (mbar_try_wait(bar, parity)) return true;
+  for (int k = 0; k < 32; ++k)
+    if (mbar_try_wait(bar, parity)) return true;
   const uint64_t limit = limit_ns ? limit_ns : 2000000000ull;
   const uint64_t t0 = global_ns();
   while (!mbar_try_wait(bar, parity)) {
