@@ -3,6 +3,8 @@
 // library; everything per sweep runs on the device from integer tables built from them.
 #include "host_tables.h"
 
+#include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdint>
 
@@ -29,14 +31,25 @@ static double normal_quantile_lower(double p) {
   return (std::fabs(normal_cdf(lo) - p) <= std::fabs(normal_cdf(hi) - p)) ? lo : hi;
 }
 
-void noise_levels(int kind, float* out) {
-  if (kind == 0) {  // Gaussian quantiles, exactly antisymmetric
-    for (int m = 0; m < kNoiseLevels / 2; ++m) {
+// The Gaussian levels are constants of the library (2048 bisections, 3 ms), so they are worked
+// out once per process, on first use.
+static const std::array<float, kNoiseLevels>& gaussian_levels() {
+  static const std::array<float, kNoiseLevels> table = [] {
+    std::array<float, kNoiseLevels> z{};
+    for (int m = 0; m < kNoiseLevels / 2; ++m) {  // exactly antisymmetric
       const double p = (m + 0.5) / kNoiseLevels;
       const float v = static_cast<float>(normal_quantile_lower(p));
-      out[m] = v;
-      out[kNoiseLevels - 1 - m] = -v;
+      z[m] = v;
+      z[kNoiseLevels - 1 - m] = -v;
     }
+    return z;
+  }();
+  return table;
+}
+
+void noise_levels(int kind, float* out) {
+  if (kind == 0) {
+    std::copy(gaussian_levels().begin(), gaussian_levels().end(), out);
   } else {  // uniform grid (2m - 4095) / 4096
     for (int m = 0; m < kNoiseLevels; ++m)
       out[m] = static_cast<float>((2.0 * m - (kNoiseLevels - 1)) / kNoiseLevels);
@@ -56,11 +69,17 @@ static double staircase(double x, int levels) {
 
 void activation_levels(float b_t, int imax, int act, int lut_levels, float* out) {
   const double b = static_cast<double>(b_t);
-  for (int I = -imax; I <= imax; ++I) {
+  for (int I = act == 0 ? 0 : -imax; I <= imax; ++I) {
     const double x = b * static_cast<double>(I);  // exact: 24-bit b times |I| < 2^20
+    if (act == 0 && x >= 10.0) {  // 1 - tanh(10) = 4e-9 < 2^-25: 1.0f from here on
+      std::fill(out + I + imax, out + 2 * imax + 1, 1.0f);
+      break;
+    }
     const double tau = (act == 0) ? std::tanh(x) : staircase(x, lut_levels);
     out[I + imax] = static_cast<float>(tau);
   }
+  if (act == 0)  // tanh is odd, in the C library bit for bit
+    for (int I = 1; I <= imax; ++I) out[imax - I] = -out[imax + I];
 }
 
 float scaled_beta(float beta, double c) {

@@ -485,6 +485,26 @@ std::string schedule_key(int steps, const float* beta, const float* eta, float x
   return k;
 }
 
+// Runs fn(begin, end) over [0, count) in contiguous parts on up to 16 host threads, at
+// least `grain` items per thread; small jobs (`work` < 2M elements) stay on the calling
+// thread, where spawning threads would cost more than it saves.
+template <class F>
+void parallel_for(int count, F fn, int grain = 64, size_t work = SIZE_MAX) {
+  const int hw = static_cast<int>(std::thread::hardware_concurrency());
+  const int nth = work < (2u << 20) ? 1 : std::max(1, std::min({hw, 16, count / grain}));
+  if (nth == 1) {
+    fn(0, count);
+    return;
+  }
+  std::vector<std::thread> th;
+  const int per = (count + nth - 1) / nth;
+  for (int k = 0; k < nth; ++k) {
+    const int b = k * per, e = std::min(count, b + per);
+    if (b < e) th.emplace_back(fn, b, e);
+  }
+  for (auto& t : th) t.join();
+}
+
 int build_schedule(std::shared_ptr<Schedule>& out, int steps, const float* beta,
                    const float* eta, float xi, int noise, int act, int lut, double c, int imax,
                    int device) {
@@ -495,8 +515,10 @@ int build_schedule(std::shared_ptr<Schedule>& out, int steps, const float* beta,
   const int width = 2 * imax + 1;
   s->stride_words = (width + 3) & ~3;
   std::vector<float> tau(static_cast<size_t>(steps) * width);
-  for (int t = 0; t < steps; ++t)
-    activation_levels(scaled_beta(beta[t], c), imax, act, lut, &tau[static_cast<size_t>(t) * width]);
+  parallel_for(steps, [&](int t0, int t1) {
+    for (int t = t0; t < t1; ++t)
+      activation_levels(scaled_beta(beta[t], c), imax, act, lut, &tau[static_cast<size_t>(t) * width]);
+  }, 16, tau.size() * 8);  // a value costs about eight of parallel_for's elements
   std::vector<float> z(kNoiseLevels);
   noise_levels(noise == PIM_NOISE_GAUSS ? 0 : 1, z.data());
   float *d_tau = nullptr, *d_eta = nullptr, *d_z = nullptr;
@@ -597,26 +619,6 @@ PIM_API int pim_activation_levels(float b_t, int imax, int act_kind, int lut_lev
 }
 
 namespace {
-
-// Runs fn(begin, end) over [0, count) in contiguous parts on up to 16 host threads, at
-// least `grain` items per thread; small jobs (`work` < 2M elements) stay on the calling
-// thread, where spawning threads would cost more than it saves.
-template <class F>
-void parallel_for(int count, F fn, int grain = 64, size_t work = SIZE_MAX) {
-  const int hw = static_cast<int>(std::thread::hardware_concurrency());
-  const int nth = work < (2u << 20) ? 1 : std::max(1, std::min({hw, 16, count / grain}));
-  if (nth == 1) {
-    fn(0, count);
-    return;
-  }
-  std::vector<std::thread> th;
-  const int per = (count + nth - 1) / nth;
-  for (int k = 0; k < nth; ++k) {
-    const int b = k * per, e = std::min(count, b + per);
-    if (b < e) th.emplace_back(fn, b, e);
-  }
-  for (auto& t : th) t.join();
-}
 
 // First (row-major order) position (i, j), i < j, where a[i*n+j] != a[j*n+i], or (-1, -1).
 // Compares 64 x 64 tiles against their transposes so both reads stay cache-friendly.
