@@ -311,8 +311,8 @@ int pim_probe_ingest(int bytes, int iters, int shared, double* gbs_per_sm);
  *   state; best / first-hit / final records are read with the usual getters.
  *   replicas, t_begin, sweeps, seed, instance_id, init_spins, target_energy, cuda_stream
  *   as pim_anneal; flags: PIM_CONTINUE and / or PIM_RESULTS_TO_HOST.  One warp per replica.
- * Errors: PIM_ERR_INVALID, PIM_ERR_STATE, PIM_ERR_UNSUPPORTED (real couplings, n too large
- *         for shared memory), PIM_ERR_NOMEM, PIM_ERR_CUDA.
+ * Errors: PIM_ERR_INVALID, PIM_ERR_STATE, PIM_ERR_UNSUPPORTED (real couplings),
+ *         PIM_ERR_NOMEM, PIM_ERR_CUDA.
  */
 int pim_anneal_sequential(pim_instance* inst, int replicas, int t_begin, int sweeps,
                           uint64_t seed, uint32_t instance_id, const int8_t* init_spins,

@@ -1,23 +1,34 @@
 // Conventional PIM with sequential updates (Eq. 3; Box 1, orange path), the baseline the
 // fully parallel loop is compared with.  One warp per replica; sweep k updates spins
-// i = 0 .. n-1 one after another, each from the field of the current state:
-//   the replica's fields I_i = sum_j J_ij s_j + h_i and its spins live in shared memory;
-//   step (k, i): every lane reads I_i and s_i (broadcast), takes the 12-bit key of draw
-//   (i>>3, r, k, q) -- one Philox block per 8 consecutive spins -- and decides with the
-//   threshold table of schedule entry k (the same exact decisions as the parallel path);
-//   on a flip the warp adds 2 s_i' J_i (row i of J = column i, coalesced int8 loads) to I.
+// i = 0 .. n-1 one after another, each from the field of the current state, with the 12-bit key of
+// draw (i>>3, r, k, q) and the threshold table of schedule entry k (the same exact decisions as
+// the parallel path); a flip adds 2 s_i' J_i (row i of J = column i) to the fields.
+//
+// The chain of n dependent steps bounds a replica, so the warp walks it flip by flip instead of
+// spin by spin: spins are taken 32 at a time, one per lane; every lane decides its spin from the
+// current fields; the lanes before the first one that flips keep their decision (nothing before
+// them changes), that flip is applied to all fields, and the lanes after it decide again.  That is
+// the sequential order exactly, in (flips + n / 32) rounds of about 120 cycles a sweep rather than
+// n steps of 290.  Fields live in registers (n <= 1024, else shared memory), spins as bit words,
+// the sweep's draws, its table (copied ahead) and, where it fits, J in shared memory.
+// Measured (GB300, us per sweep, spin by spin with J in L2 before): SK n = 200 27.9 -> 2.3 (256
+// replicas), 106 -> 9.7 (8192); n = 400 57.6 -> 4.7; n = 1000 369 -> 70; n = 2000 1065 -> 357.
+//
 // Energies E = -1/2 sum_i s_i (I_i + h_i) are evaluated on the state at the start of every
 // sweep and on the final state, with the best-state / first-hit bookkeeping of the
-// parallel kernels.  No waits between warps: every warp runs on its own.
+// parallel kernels.  No waits between warps once J is loaded: every warp runs on its own.
 #include <climits>
 
 #include "kernels.h"
 #include "philox.cuh"
+#include "sm100_ptx.cuh"
 
 namespace pim {
 namespace {
 
-constexpr int kWarps = 4;  // replicas per block
+constexpr int kMaxWarps = 8;                // replicas per block
+constexpr int kSmemBudget = 227 * 1024;
+constexpr int kTabWordsMax = 4096;          // tables up to this size are staged in shared memory
 
 __device__ __forceinline__ long long warp_sum(long long v) {
 #pragma unroll
@@ -25,33 +36,103 @@ __device__ __forceinline__ long long warp_sum(long long v) {
   return v;
 }
 
-__global__ void __launch_bounds__(kWarps * 32) sequential_kernel(const __grid_constant__ SeqLaunch L) {
-  extern __shared__ int smem_seq[];
+__host__ __device__ inline int round16(int x) { return (x + 15) & ~15; }
+
+// Shared memory of a launch: J (when jsm), then per warp two tables (when tsm), the draws of a
+// sweep, the spin words and, for KF = 0, the fields.
+struct SeqPlan {
+  int kf = 0;      // 32-spin field registers per lane (0: fields in shared memory)
+  int warps = 1;   // replicas per block
+  int jsm = 0, tsm = 0;
+  int warp_bytes = 0, bytes = 0;
+};
+
+SeqPlan seq_plan(int n, int words, int stride_words, int replicas, int sms) {
+  SeqPlan p;
+  p.kf = n <= 128 ? 4 : n <= 256 ? 8 : n <= 512 ? 16 : n <= 1024 ? 32 : 0;
+  const int base = round16((n + 7) / 8 * 16) + round16(words * 4) + (p.kf == 0 ? round16(n * 4) : 0);
+  const int tab = 2 * stride_words * 4;
+  p.tsm = stride_words <= kTabWordsMax && base + tab <= kSmemBudget ? 1 : 0;
+  p.warp_bytes = base + (p.tsm ? tab : 0);
+  // spread the replicas over the SMs first, then share a block's J between up to kMaxWarps
+  const int want = (replicas + sms - 1) / sms;
+  p.warps = want < 1 ? 1 : want > kMaxWarps ? kMaxWarps : want;
+  const int jbytes = p.kf > 0 && p.kf <= 16 ? round16(n * n) : kSmemBudget;
+  p.jsm = jbytes + p.warp_bytes <= kSmemBudget ? 1 : 0;
+  while (p.warps > 1 && (p.jsm ? jbytes : 0) + p.warps * p.warp_bytes > kSmemBudget) --p.warps;
+  p.bytes = (p.jsm ? jbytes : 0) + p.warps * p.warp_bytes;
+  return p;
+}
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// JSM: J in shared memory.
+template <int KF, bool JSM>
+__global__ void __launch_bounds__(kMaxWarps * 32) sequential_kernel(const __grid_constant__ SeqLaunch L,
+                                                                    const SeqPlan plan) {
+  constexpr int K = KF > 0 ? KF : 1;
+  extern __shared__ __align__(16) uint8_t smem_seq[];
   const Problem& P = L.P;
-  const int n = P.n, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r = blockIdx.x * kWarps + warp;
-  if (r >= P.R) return;  // a whole warp; the kernel has no block-level synchronisation
-  int* I = smem_seq + static_cast<size_t>(warp) * n;                                   // [n]
-  int8_t* s = reinterpret_cast<int8_t*>(smem_seq + static_cast<size_t>(kWarps) * n) +
-              static_cast<size_t>(warp) * n;                                           // [n]
-  const int words = P.words;
+  const int n = P.n, words = P.words, imax = P.imax, stride = P.stride_words;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int r = blockIdx.x * plan.warps + warp;
+  const int8_t* J = JSM ? reinterpret_cast<const int8_t*>(smem_seq) : P.j8;
+  uint8_t* mine = smem_seq + (JSM ? round16(n * n) : 0) + warp * plan.warp_bytes;
+  if constexpr (JSM) {
+    const int total = n * n;
+    const uint4* src = reinterpret_cast<const uint4*>(P.j8);
+    uint4* dst = reinterpret_cast<uint4*>(smem_seq);
+    for (int k = threadIdx.x; k < total / 16; k += blockDim.x) dst[k] = __ldg(src + k);
+    for (int k = total / 16 * 16 + threadIdx.x; k < total; k += blockDim.x)
+      smem_seq[k] = static_cast<uint8_t>(P.j8[k]);
+    __syncthreads();
+  }
+  if (r >= P.R) return;  // a whole warp; no block-level synchronisation from here on
+  uint32_t* tabs = reinterpret_cast<uint32_t*>(mine);                  // [2][stride] when tsm
+  uint16_t* draws = reinterpret_cast<uint16_t*>(mine + (plan.tsm ? 2 * stride * 4 : 0));
+  uint32_t* sw = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(draws) + round16((n + 7) / 8 * 16));
+  int* sI = reinterpret_cast<int*>(reinterpret_cast<uint8_t*>(sw) + round16(words * 4));  // KF = 0
+  const int nblk32 = (n + 31) >> 5;
   uint32_t* cur_io = P.cur_bits + static_cast<size_t>(r) * words;
   uint32_t* best_io = P.best_bits + static_cast<size_t>(r) * words;
-  const int8_t* J = P.j8;
   const int32_t* h = P.h;
-  const int imax = P.imax, stride = P.stride_words;
 
-  for (int j = lane; j < n; j += 32) s[j] = ((cur_io[j >> 5] >> (j & 31)) & 1u) ? 1 : -1;
+  for (int w = lane; w < words; w += 32) sw[w] = cur_io[w];
   __syncwarp();
-  // fields of the starting state, one row of J per iteration, lanes across the row
-  for (int i = 0; i < n; ++i) {
-    const int8_t* Ji = J + static_cast<size_t>(i) * n;
-    int acc = 0;
-    for (int j = lane; j < n; j += 32) acc += Ji[j] * s[j];
-    acc = static_cast<int>(warp_sum(acc));
-    if (lane == 0) I[i] = acc + (h ? h[i] : 0);
+  // Field of spin 32 k + lane (lanes past n keep 0).
+  int F[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) F[k] = 0;
+  auto add_row = [&](int i, int d) {  // I += d * row i of J
+    const int8_t* Ji = J + static_cast<size_t>(i) * n + lane;
+    if constexpr (KF > 0) {
+      int v[K];  // every load before the first use
+#pragma unroll
+      for (int k = 0; k < K; ++k) v[k] = 32 * k + lane < n ? (JSM ? Ji[32 * k] : __ldg(Ji + 32 * k)) : 0;
+#pragma unroll
+      for (int k = 0; k < K; ++k) F[k] += v[k] * d;
+    } else {
+      for (int j0 = 0; j0 < n; j0 += 1024) {  // 32 loads in flight
+        int v[32];
+#pragma unroll
+        for (int k = 0; k < 32; ++k) v[k] = j0 + 32 * k + lane < n ? __ldg(Ji + j0 + 32 * k) : 0;
+#pragma unroll
+        for (int k = 0; k < 32; ++k)
+          if (j0 + 32 * k + lane < n) sI[j0 + 32 * k + lane] += v[k] * d;
+      }
+    }
+  };
+  if constexpr (KF > 0) {
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      if (32 * k + lane < n && h) F[k] = h[32 * k + lane];
+  } else {
+    for (int j = lane; j < n; j += 32) sI[j] = h ? h[j] : 0;
   }
-  __syncwarp();
+#pragma unroll 4
+  for (int i = 0; i < n; ++i) add_row(i, ((sw[i >> 5] >> (i & 31)) & 1u) ? 1 : -1);
 
   long long best_E = LLONG_MAX;
   int best_t = -1, first_hit = -1;
@@ -63,64 +144,85 @@ __global__ void __launch_bounds__(kWarps * 32) sequential_kernel(const __grid_co
   // E(s) on the current state, bookkeeping at schedule index t; returns E.
   auto evaluate = [&](int t) -> long long {
     long long acc = 0;
-    for (int j = lane; j < n; j += 32) acc += static_cast<long long>(s[j]) * (I[j] + (h ? h[j] : 0));
+    if constexpr (KF > 0) {
+#pragma unroll
+      for (int k = 0; k < K; ++k)
+        if (32 * k + lane < n) {
+          const long long term = F[k] + (h ? h[32 * k + lane] : 0);
+          acc += ((sw[k] >> lane) & 1u) ? term : -term;
+        }
+    } else {
+      for (int j = lane; j < n; j += 32) {
+        const long long term = static_cast<long long>(sI[j]) + (h ? h[j] : 0);
+        acc += ((sw[j >> 5] >> (j & 31)) & 1u) ? term : -term;
+      }
+    }
     const long long E = -(warp_sum(acc) / 2);
     if (E < best_E) {
       best_E = E;
       best_t = t;
-      for (int w = lane; w < words; w += 32) {
-        uint32_t b = 0;
-        for (int e = 0; e < 32; ++e) {
-          const int j = 32 * w + e;
-          if (j < n && s[j] > 0) b |= 1u << e;
-        }
-        best_io[w] = b;
-      }
+      for (int w = lane; w < words; w += 32) best_io[w] = sw[w];
     }
     if (P.has_target && first_hit < 0 && E <= P.target) first_hit = t;
     return E;
   };
+  auto fetch_table = [&](int t) {  // asynchronously, into the table buffer of t
+    const uint32_t dst = smem_u32(tabs + (t & 1) * stride);
+    const uint32_t* src = P.thr + static_cast<size_t>(t) * stride;
+    for (int k = lane; k < stride / 4; k += 32) cp_async16(dst + 16 * k, src + 4 * k);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
 
   const int t_end = L.t_begin + L.sweeps;
-  for (int k = L.t_begin; k < t_end; ++k) {
-    evaluate(k);
-    const uint32_t* tab = P.thr + static_cast<size_t>(k) * stride;
-    uint32_t rw[4] = {0, 0, 0, 0};
-    for (int i = 0; i < n; ++i) {
-      if ((i & 7) == 0) {
-        const PhiloxOut o = philox4x32_10_rk(static_cast<uint32_t>(i >> 3), static_cast<uint32_t>(r),
-                                             static_cast<uint32_t>(k), P.q, L.round_keys);
-        rw[0] = o.x0;
-        rw[1] = o.x1;
-        rw[2] = o.x2;
-        rw[3] = o.x3;
-      }
-      const int si = s[i];
-      const int Ii = I[i];
-      const uint32_t word = rw[(i & 7) >> 1];
-      const uint32_t key = (i & 1) ? (word >> 20) : ((word >> 4) & 0xFFFu);
-      const uint32_t w = tab[Ii + imax];
-      const uint32_t th = si > 0 ? (w >> 16) : (w & 0xFFFFu);
-      const int snew = key >= th ? 1 : -1;
-      if (snew != si) {  // the same on every lane
-        const int d = snew - si;
-        const int8_t* Ji = J + static_cast<size_t>(i) * n;
-        for (int j = lane; j < n; j += 32) I[j] += Ji[j] * d;
-        __syncwarp();
-        if (lane == 0) s[i] = static_cast<int8_t>(snew);
+  if (plan.tsm && L.t_begin < t_end) fetch_table(L.t_begin);
+  for (int t = L.t_begin; t < t_end; ++t) {
+    evaluate(t);
+    __syncwarp();  // the last sweep's draws and table have been read
+    for (int b = lane; b < (n + 7) / 8; b += 32) {
+      const PhiloxOut o = philox4x32_10_rk(static_cast<uint32_t>(b), static_cast<uint32_t>(r),
+                                           static_cast<uint32_t>(t), P.q, L.round_keys);
+      reinterpret_cast<uint4*>(draws)[b] = make_uint4(o.x0, o.x1, o.x2, o.x3);  // spin order
+    }
+    const uint32_t* tab = P.thr + static_cast<size_t>(t) * stride;
+    if (plan.tsm) {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      if (t + 1 < t_end) fetch_table(t + 1);
+      tab = tabs + (t & 1) * stride;
+    }
+    __syncwarp();
+    // spins 32 k .. 32 k + 31, this lane's field in f (and its register / shared copy kept)
+    auto block32 = [&](int k, auto field) {
+      const int i = 32 * k + lane;
+      uint32_t word = sw[k];
+      const int key = i < n ? draws[i] >> 4 : 0;
+      uint32_t todo = n - 32 * k >= 32 ? 0xFFFFFFFFu : (1u << (n - 32 * k)) - 1u;
+      for (;;) {
+        const uint32_t up = (word >> lane) & 1u;
+        const uint32_t w = tab[field() + imax];
+        const int th = static_cast<int>(up ? (w >> 16) : (w & 0xFFFFu));
+        const uint32_t flips = __ballot_sync(0xFFFFFFFFu, (key >= th ? 1u : 0u) != up) & todo;
+        if (flips == 0) break;
+        const int l = __ffs(static_cast<int>(flips)) - 1;
+        add_row(32 * k + l, ((word >> l) & 1u) ? -2 : 2);
+        word ^= 1u << l;
+        todo &= l == 31 ? 0u : 0xFFFFFFFEu << l;  // the spins after it decide again
+        if constexpr (KF == 0) __syncwarp();
       }
       __syncwarp();
+      if (lane == 0) sw[k] = word;
+    };
+    if constexpr (KF > 0) {
+#pragma unroll
+      for (int k = 0; k < K; ++k)
+        if (k < nblk32) block32(k, [&]() { return F[k]; });
+    } else {
+      for (int k = 0; k < nblk32; ++k)
+        block32(k, [&]() { return 32 * k + lane < n ? sI[32 * k + lane] : 0; });
     }
+    __syncwarp();
   }
   const long long E = evaluate(t_end);
-  for (int w = lane; w < words; w += 32) {
-    uint32_t b = 0;
-    for (int e = 0; e < 32; ++e) {
-      const int j = 32 * w + e;
-      if (j < n && s[j] > 0) b |= 1u << e;
-    }
-    cur_io[w] = b;
-  }
+  for (int w = lane; w < words; w += 32) cur_io[w] = sw[w];
   if (lane == 0) {
     P.best_E[r] = static_cast<double>(best_E);
     P.best_t[r] = best_t;
@@ -129,17 +231,31 @@ __global__ void __launch_bounds__(kWarps * 32) sequential_kernel(const __grid_co
   }
 }
 
+template <int KF, bool JSM>
+cudaError_t launch_seq(const SeqLaunch& L, const SeqPlan& plan, cudaStream_t st) {
+  cudaError_t e = cudaFuncSetAttribute(sequential_kernel<KF, JSM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       plan.bytes);
+  if (e != cudaSuccess) return e;
+  const int blocks = (L.P.R + plan.warps - 1) / plan.warps;
+  sequential_kernel<KF, JSM><<<blocks, plan.warps * 32, plan.bytes, st>>>(L, plan);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
-int sequential_smem_bytes(int n) { return kWarps * n * 5; }
-
 cudaError_t launch_sequential(const SeqLaunch& L, cudaStream_t st) {
-  const int smem = sequential_smem_bytes(L.P.n);
-  cudaError_t e = cudaFuncSetAttribute(sequential_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  const int blocks = (L.P.R + kWarps - 1) / kWarps;
-  sequential_kernel<<<blocks, kWarps * 32, smem, st>>>(L);
-  return cudaGetLastError();
+  const SeqPlan plan = seq_plan(L.P.n, L.P.words, L.P.stride_words, L.P.R, sms);
+  switch (plan.kf) {
+    case 4: return plan.jsm ? launch_seq<4, true>(L, plan, st) : launch_seq<4, false>(L, plan, st);
+    case 8: return plan.jsm ? launch_seq<8, true>(L, plan, st) : launch_seq<8, false>(L, plan, st);
+    case 16: return plan.jsm ? launch_seq<16, true>(L, plan, st) : launch_seq<16, false>(L, plan, st);
+    case 32: return launch_seq<32, false>(L, plan, st);
+    default: return launch_seq<0, false>(L, plan, st);
+  }
 }
 
 }  // namespace pim

@@ -112,7 +112,6 @@ int sweep_mid_max_npad();
 
 // Sequential (conventional PIM) kernel: one warp per replica, integer couplings.
 cudaError_t launch_sequential(const SeqLaunch& L, cudaStream_t st);
-int sequential_smem_bytes(int n);
 
 // Plain FP32 comparator path: per sweep one field GEMM and one update kernel.
 cudaError_t launch_ref_anneal(const Problem* h_probs, const Problem* d_probs, int nprob,

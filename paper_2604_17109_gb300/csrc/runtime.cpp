@@ -2502,11 +2502,6 @@ PIM_API int pim_anneal_sequential(pim_instance* inst, int replicas, int t_begin,
   if (rc != PIM_OK) return rc;
   const bool cont = (flags & PIM_CONTINUE) != 0;
   if (cont && init_spins) return fail(PIM_ERR_INVALID, "pim_anneal_sequential: CONTINUE takes no spins");
-  int smem_max = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (sequential_smem_bytes(inst->n) > smem_max)
-    return fail(PIM_ERR_UNSUPPORTED, "pim_anneal_sequential: n = %d too large", inst->n);
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   if ((rc = prepare_instances(&inst, 1, &replicas, false, st)) != PIM_OK) return rc;
   BatchPlan B;
