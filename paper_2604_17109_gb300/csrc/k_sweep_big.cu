@@ -35,6 +35,7 @@
 
 #include "kernels.h"
 #include "philox.cuh"
+#include "real_rule.cuh"
 #include "sm100_ptx.cuh"
 
 namespace pim {
@@ -45,6 +46,8 @@ constexpr int kTabWords = 8192;     // threshold table of one step staged in sha
 constexpr int kEpiWarps = 16;
 constexpr int kThreads = (2 + kEpiWarps) * 32;
 constexpr int kSmemBudget = 227 * 1024;
+constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23: integer D (|D| < 2^22) in the low mantissa bits
+constexpr uint32_t kMagicBits = 0x4B400000u;
 
 // K-blocks per ring stage.  A bulk copy costs about 0.16 us of the producer's time whatever
 // its size (up to 16 KB measured), so a stage moves two K-blocks of the tile's spins in one
@@ -459,82 +462,129 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_big_kernel(const __grid_con
       if (cb == 0 && epi && grp == 0) __stcg(&energy[((t - t_begin + 1) % 3) * rpad + rl], EAcc(0));
       EAcc eacc = 0;
       uint32_t nxt = 0;
-      const bool tab_in_smem = !REAL && tab_smem;
       if (epi) {
         // While the MMAs run: the bookkeeping of s(t-1), whose energy the last barrier
         // completed, and this step's thresholds staged (the previous step's reads ended
         // before that barrier); then sync the 16 epilogue warps.
         if (t > t_begin) track(t - 1, prev);
-        if (tab_in_smem && !last) {
+        if (!REAL && tab_smem && !last) {
           const uint4* src =
               reinterpret_cast<const uint4*>(P.thr + static_cast<size_t>(t) * P.stride_words);
           for (int k = tid - 64; k < P.stride_words / 4; k += kEpiWarps * 32)
             reinterpret_cast<uint4*>(sTab)[k] = __ldg(src + k);
         }
         asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory");
-        const bool ok = mbar_wait_fast(bar_done, done_phase, L.wait_ns);
-        if (!ok) {
+        // The sweep's noise while the MMAs run: draws (integer couplings) or xi s + eta z (real).
+        uint32_t rw[kSPT / 2];
+        float ns[REAL ? kSPT : 1];
+        float b = 0.0f, eta = 0.0f;
+        if (warp_active && !last) {
+          if constexpr (REAL) {
+            b = P.sched_b[t];
+            eta = P.sched_eta[t];
+          }
+#pragma unroll
+          for (int k = 0; k < kSPT / 8; ++k) {
+            const PhiloxOut o = philox4x32_10_rk(static_cast<uint32_t>((col0 >> 3) + k), static_cast<uint32_t>(r),
+                                                 static_cast<uint32_t>(t), P.q, L.round_keys);
+            rw[4 * k] = o.x0, rw[4 * k + 1] = o.x1, rw[4 * k + 2] = o.x2, rw[4 * k + 3] = o.x3;
+          }
+          if (REAL && P.act == 0)
+#pragma unroll
+            for (int e = 0; e < (REAL ? kSPT : 0); ++e) {
+              const uint32_t word = rw[e >> 1];
+              const uint32_t key = (e & 1) ? (word >> 20) : ((word >> 4) & 0xFFFu);
+              ns[e] = __fmaf_rn(eta, sZ[key], ((cur >> e) & 1u) ? P.xi : -P.xi);
+            }
+        }
+        const bool ok = __all_sync(0xFFFFFFFFu, mbar_wait_fast(bar_done, done_phase, L.wait_ns));
+        if (!ok && lane == 0) {
           atomicOr(L.err, kDevErrTimeout);
           grid_abort(L.bar);
         }
         tc_fence_after();
-        if (warp_active) {
-          const uint32_t* tab = nullptr;
-          float b = 0.0f, eta = 0.0f;
-          float* dump = nullptr;  // diagnostics: fields of the first sweep (real couplings)
-          if (REAL && P.fields_out != nullptr && t == t_begin && !last && row_valid)
-            dump = P.fields_out + static_cast<size_t>(r) * n + col0;
-          if constexpr (REAL) {
-            if (!last) {
-              b = P.sched_b[t];
-              eta = P.sched_eta[t];
-            }
-          } else {
-            tab = tab_in_smem ? sTab : P.thr + static_cast<size_t>(last ? t_begin : t) * P.stride_words;
-          }
+        if (warp_active && ok) {
+          const bool dumps = REAL && P.fields_out != nullptr && t == t_begin && !last && row_valid;
+          const uint32_t ta = tmem + (static_cast<uint32_t>(quad * 32) << 16) + grp * kSPT;
 #pragma unroll
           for (int c = 0; c < kChunks; ++c) {
             uint32_t v[16];
-            tmem_ld16(tmem + (static_cast<uint32_t>(quad * 32) << 16) + grp * kSPT + 16 * c, v);
-            PhiloxOut o0{}, o1{};
-            if (!last) {
-              const uint32_t ctr = static_cast<uint32_t>((col0 + 16 * c) >> 3);
-              o0 = philox4x32_10_rk(ctr, static_cast<uint32_t>(r), static_cast<uint32_t>(t), P.q,
-                                    L.round_keys);
-              o1 = philox4x32_10_rk(ctr + 1u, static_cast<uint32_t>(r), static_cast<uint32_t>(t),
-                                    P.q, L.round_keys);
-            }
+            tmem_ld16(ta + 16 * c, v);
             tmem_wait_ld(v);
-            const uint32_t rw[8] = {o0.x0, o0.x1, o0.x2, o0.x3, o1.x0, o1.x1, o1.x2, o1.x3};
+            const uint32_t cw16 = (cur >> (16 * c)) & 0xFFFFu;
+            if constexpr (REAL) {
+              float x[16];
 #pragma unroll
-            for (int e = 0; e < 16; ++e) {
-              const int bit = 16 * c + e;
-              const uint32_t s = (cur >> bit) & 1u;
-              const uint32_t word = rw[e >> 1];
-              const uint32_t key = (e & 1) ? (word >> 20) : ((word >> 4) & 0xFFFu);
-              if constexpr (REAL) {
-                const float hv = __uint_as_float(sH[grp * kSPT + bit]);
-                const float I = __fadd_rn(__uint_as_float(v[e]), hv);
-                if (dump != nullptr && col0 + bit < n) dump[bit] = I;
-                const float term = __fadd_rn(I, hv);
-                eacc += s ? term : -term;
-                if (!last) {
-                  const float x = __fmul_rn(b, I);
-                  const float tau = P.act == 0 ? tanhf(x) : staircase(x, P.lut_levels);
-                  const float a = __fadd_rn(tau, s ? P.xi : -P.xi);
-                  const float delta = __fadd_rn(a, __fmul_rn(eta, sZ[key]));
-                  nxt |= (delta >= 0.0f ? 1u : 0u) << bit;
+              for (int e = 0; e < 16; ++e) {
+                const float hv = __uint_as_float(sH[grp * kSPT + 16 * c + e]);
+                x[e] = __fadd_rn(__uint_as_float(v[e]), hv);
+                const float term = __fadd_rn(x[e], hv);
+                eacc += ((cw16 >> e) & 1u) ? term : -term;
+              }
+              if (dumps)  // diagnostics: fields of the first sweep
+#pragma unroll
+                for (int e = 0; e < 16; ++e)
+                  if (col0 + 16 * c + e < n) P.fields_out[static_cast<size_t>(r) * n + col0 + 16 * c + e] = x[e];
+              if (!last) {
+                float g[16], least = P.act == 0 ? 8.0f : 0.0f;
+                const float margin = rule_margin(P.act, P.xi);
+#pragma unroll
+                for (int e = 0; e < 16; ++e) x[e] = __fmul_rn(b, x[e]);
+                if (P.act == 0) {
+#pragma unroll
+                  for (int e = 0; e < 16; ++e) {
+                    g[e] = __fadd_rn(tanh_approx(x[e]), ns[REAL ? 16 * c + e : 0]);
+                    least = fminf(least, fabsf(g[e]));
+                  }
                 }
-              } else {
-                const int hv = static_cast<int>(sH[grp * kSPT + bit]);
-                const int I = __float2int_rn(__uint_as_float(v[e])) + hv;
-                const int term = I + hv;
-                eacc += s ? term : -term;
-                if (!last) {
-                  const uint32_t w = tab[I + P.imax];
-                  const uint32_t th = s ? (w >> 16) : (w & 0xFFFFu);
-                  nxt |= (key >= th ? 1u : 0u) << bit;
+                if (__any_sync(0xFFFFFFFFu, least <= margin))
+                  settle_chunk<16>(g, x, static_cast<uint32_t>((col0 + 16 * c) >> 3), static_cast<uint32_t>(r),
+                                   static_cast<uint32_t>(t), P.q, L.round_keys, cw16, margin, P.xi, eta, P.act,
+                                   P.lut_levels, sZ);
+                uint32_t neg = 0;
+#pragma unroll
+                for (int e = 15; e >= 0; --e) neg = __funnelshift_l(__float_as_uint(g[e]), neg, 1);
+                nxt |= (~neg & 0xFFFFu) << (16 * c);
+              }
+            } else {
+              // bits of (D + 1.5 * 2^23) + h = 0x4B400000 + I; the 16-bit threshold of (s, I) is
+              // half s of the table's word I + imax, and key >= M <=> draw - 16 M >= 0
+              uint32_t vb[16];
+#pragma unroll
+              for (int e = 0; e < 16; ++e) {
+                const int hv = static_cast<int>(sH[grp * kSPT + 16 * c + e]);
+                vb[e] = __float_as_uint(__fadd_rn(__uint_as_float(v[e]), kMagic)) + hv;
+                const int term = static_cast<int>(vb[e] - kMagicBits) + hv;
+                eacc += ((cw16 >> e) & 1u) ? term : -term;
+              }
+              if (!last) {
+                uint32_t neg = 0;
+                auto decide = [&](int e, uint32_t th) {
+                  const uint32_t word = rw[8 * c + (e >> 1)];
+                  const uint32_t d = (e & 1) ? (word >> 16) : (word & 0xFFFFu);
+                  neg = __funnelshift_l(d + th * 0xFFFFFFF0u, neg, 1);
+                };
+                if (tab_smem) {
+                  const uint32_t tab_c = smem_u32(sTab) + 4u * static_cast<uint32_t>(P.imax) - 4u * kMagicBits;
+#pragma unroll
+                  for (int e = 15; e >= 0; --e) {
+                    uint32_t th;
+                    asm volatile("ld.shared.u16 %0, [%1];"
+                                 : "=r"(th)
+                                 : "r"(tab_c + 4u * vb[e] + 2u * ((cw16 >> e) & 1u)));
+                    decide(e, th);
+                  }
+                } else {  // through L1
+                  const uint16_t* tab16 = reinterpret_cast<const uint16_t*>(
+                      P.thr + static_cast<size_t>(t) * P.stride_words + P.imax);
+                  uint32_t th[16];
+#pragma unroll
+                  for (int e = 0; e < 16; ++e)
+                    th[e] = __ldg(tab16 + 2 * static_cast<int>(vb[e] - kMagicBits) + static_cast<int>((cw16 >> e) & 1u));
+#pragma unroll
+                  for (int e = 15; e >= 0; --e) decide(e, th[e]);
                 }
+                nxt |= (~neg & 0xFFFFu) << (16 * c);
               }
             }
           }

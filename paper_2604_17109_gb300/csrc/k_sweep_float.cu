@@ -24,7 +24,7 @@
 //    of the columns) and one MMA warp, coupled by mbarriers; two accumulators, so that the
 //    energy of s(t) is summed while s(t+1) is decided and multiplied.
 //  - The noise is drawn while the MMAs run.
-//  - tanh is the hardware's approximation first: where the sum it gives lies within kMargin of
+//  - tanh is the hardware's approximation first: where the sum it gives lies within a margin of
 //    zero, the decision is taken by the rule above instead (about one spin in 30 000), so every
 //    decision is the rule's own.
 // Measured (GB300, us per sweep) against 128-lane tiles with the rule unrolled for every column
@@ -39,10 +39,10 @@
 //   n = sat(trunc(Q(eta_t) Q(z) / 2^F)), s' = +1 iff sat(a + n) >= 0,
 // and the energy is summed exactly in integers.
 #include <cfloat>
-#include <cmath>
 
 #include "kernels.h"
 #include "philox.cuh"
+#include "real_rule.cuh"
 #include "sm100_ptx.cuh"
 
 namespace pim {
@@ -124,33 +124,6 @@ struct FloatCfg {
 template <int CAP>
 int float_smem_bytes(bool fixed) {
   return FloatCfg<CAP>::kFixed + (fixed ? 2 : 1) * FloatCfg<CAP>::kJBytes;
-}
-
-// |tanh.approx(x) - tanhf(x)| <= 8.0e-6 on sm_103a, measured over every float (documented: 2^-11
-// relative); kMargin is five times that.  The FP32 roundings of xi s + eta z and of the rule's
-// own sums are below 1e-6 (1 + xi) each near zero and are covered where the margin is used.
-constexpr float kMargin = 4e-5f;
-
-__device__ __forceinline__ float tanh_approx(float x) {
-  float y;
-  asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-// The rule of the header for the spins of a chunk with |g| <= margin: g = +1 or -1 from
-// x = b I, the draws rw and the old spins ob.  Out of line: the common path keeps its registers.
-template <int W>
-__device__ __noinline__ void rule_chunk(float* g, const float* x, const uint32_t* rw, uint32_t ob, float margin,
-                                        float xi, float eta, int act, int levels, const float* sZ) {
-#pragma unroll 1
-  for (int e = 0; e < W; ++e) {
-    if (!(fabsf(g[e]) <= margin)) continue;
-    const uint32_t word = rw[e >> 1];
-    const float z = sZ[(e & 1) ? (word >> 20) : ((word >> 4) & 0xFFFu)];
-    const float tau = act == 0 ? tanhf(x[e]) : staircase(x[e], levels);
-    const float a = __fadd_rn(tau, ((ob >> e) & 1u) ? xi : -xi);
-    g[e] = __fadd_rn(a, __fmul_rn(eta, z)) >= 0.0f ? 1.0f : -1.0f;
-  }
 }
 
 // kPlain / kFixedPoint: CTA b runs work item b of L (one instance x L.rows replicas).
@@ -284,8 +257,7 @@ __global__ void __launch_bounds__(FloatCfg<CAP>::kBoundThreads, 1)
       // ---- decision warps -------------------------------------------------------------
       const float xi = P.xi;
       const int act = P.act, levels = P.lut_levels;
-      // (the staircase goes by the rule alone)
-      const float margin = act == 0 ? kMargin + 4e-6f * (1.0f + fabsf(xi)) : INFINITY;
+      const float margin = rule_margin(act, xi);
       float* const fields = SERVE ? nullptr : P.fields_out;
       const int nchw = nch * (16 / W);
       uint8_t* bits8 = reinterpret_cast<uint8_t*>(sBits);
@@ -418,15 +390,9 @@ __global__ void __launch_bounds__(FloatCfg<CAP>::kBoundThreads, 1)
                 g[e] = __fadd_rn(tanh_approx(x[e]), g[e]);
                 least = fminf(least, fabsf(g[e]));
               }
-              if (__any_sync(0xFFFFFFFFu, least <= margin)) {
-                float gm[W], xm[W];
-                uint32_t rm[W / 2];
-#pragma unroll
-                for (int e = 0; e < W; ++e) gm[e] = g[e], xm[e] = x[e], rm[e / 2] = rw[e / 2];
-                rule_chunk<W>(gm, xm, rm, ob, margin, xi, eta, act, levels, sZ);
-#pragma unroll
-                for (int e = 0; e < W; ++e) g[e] = gm[e];
-              }
+              if (__any_sync(0xFFFFFFFFu, least <= margin))
+                settle_chunk<W>(g, x, c * W / 8, static_cast<uint32_t>(rg), static_cast<uint32_t>(t), q,
+                                L.round_keys, ob, margin, xi, eta, act, levels, sZ);
             }
             // the sign of g is the sign of the BF16 spin
             uint32_t neg = 0, wd[W / 2];
