@@ -1,20 +1,21 @@
 // Large-N PIMI sweep kernel (N > 256): persistent, cooperative, one CTA per (128-replica
 // tile, NT-spin column block), all sweeps in one launch.  Three operand variants:
-//   FP8   integer couplings: FP8 E4M3 spin and coupling images (tcgen05 kind::f8f6f4), both
+//   FP8   integer couplings: FP8 E4M3 spins and couplings (tcgen05 kind::f8f6f4), the couplings
 //         streamed every sweep; exact integer fields and the exact threshold-table decision;
 //   BF16  real couplings: BF16 images (kind::f16), FP32 fields, Eq. 4 evaluated in FP32;
 //   FP4   integer couplings in {0, +-1, +-2, +-3, +-4, +-6}, NT = 64: the CTA's coupling rows
-//         stay in shared memory as packed E2M1 for the whole launch and only the E2M1 spin
-//         tile streams (block-scaled kind::mxf4 with unit scale factors, so the products and
-//         the FP32 sums stay exact integers); same decision as FP8.
+//         stay in shared memory as packed E2M1 for the whole launch (block-scaled kind::mxf4
+//         with unit scale factors, so the products and the FP32 sums stay exact integers);
+//         same decision as FP8.
 // NT (64 or 128 spins) and the variant are chosen per instance by the host.
 //
 // Per sweep t (Box 1, PIMI loop; Eq. 2 then Eq. 4):
-//   fields   D[r, i] = sum_j S[r, j] J[i, j] for the CTA's 128 replicas and NT spins: the
-//            K dimension (all N spins) streams through a shared-memory ring filled by
-//            cp.async.bulk (spins of the tile from the global spin image, two K-blocks per
-//            copy, rows of J from the coupling image unless they are resident), consumed by
-//            tcgen05.mma into TMEM.
+//   fields   D[r, i] = sum_j S[r, j] J[i, j] for the CTA's 128 replicas and NT spins, over the K
+//            dimension (all N spins) in stages: the spins come from the global bit image, expanded by
+//            the epilogue warps into tensor memory (the MMA's A operand), the rows of J from the
+//            coupling image through a shared-memory ring filled by cp.async.bulk unless they are
+//            resident.  Streaming the spins as operand bytes took as much of the L2-to-SM path as J
+//            itself, which bounded the K loop (about 10 TB/s over all SMs).
 //   decision 16 epilogue warps (4 TMEM lane quadrants x 4 column groups); each thread owns
 //            one replica and NT/4 spins for the whole anneal, keeps their old / new / best
 //            bits in registers, draws the Philox blocks and decides: integer couplings by
@@ -28,6 +29,9 @@
 //            next sweep's K-loop every CTA reads the replica energies of s(t), updates best /
 //            first hit (redundantly, identically in all CTAs) and keeps its own spins of s(t)
 //            as the best state when the energy improved.
+// Measured (GB300, us per sweep; spins streamed as operand bytes before): BF16 N = 8192 x 256
+// replicas 40.1 -> 33.8, x 64 29.7 -> 26.2; BF16 N = 2000 x 256 11.3 -> 9.8, N = 1000 x 128 7.9 -> 6.9;
+// FP8 N = 4800 x 128 10.5 -> 10.0; E2M1 N = 4096 x 256 7.0 -> 6.7 (N = 1201 x 200 4.3 -> 4.6).
 #include <algorithm>
 #include <cfloat>
 #include <climits>
@@ -49,68 +53,95 @@ constexpr int kSmemBudget = 227 * 1024;
 constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23: integer D (|D| < 2^22) in the low mantissa bits
 constexpr uint32_t kMagicBits = 0x4B400000u;
 
-// K-blocks per ring stage.  A bulk copy costs about 0.16 us of the producer's time whatever
-// its size (up to 16 KB measured), so a stage moves two K-blocks of the tile's spins in one
-// copy (the spin image is tile-major for that) instead of one copy per K-block.
-constexpr int KPS = 2;
-// Odd sweeps walk the K-blocks from the last to the first, so a sweep starts on the coupling
+// The K loop runs in stages of kPB K-blocks through a ring of kStages: the spins' operand in tensor
+// memory (32 columns, i.e. 128 bytes of every row, per K-block), expanded from the bit image by the
+// epilogue warps (warp group g takes K-block g of a stage), and the streamed coupling rows in shared
+// memory, on one full and one empty barrier.  A wait that finds its phase complete still costs the
+// MMA warp 85 cycles and a commit 25, and the tensor pipe idles meanwhile (four MMAs of N = 128 take
+// 260; 377 with two waits and two commits per K-block), so a stage is as large as both memories allow.
+constexpr int kPB = 4;
+constexpr int kStages = 3;
+constexpr int kACols = 32;
+constexpr int KPS = 2;  // K-blocks that odd sweeps keep in ascending order
+// Odd sweeps walk the K-blocks from the last pair to the first, so a sweep starts on the coupling
 // blocks the previous one read last, which are still in L2 (BF16 Max-Cut N = 8192, whose
-// 134 MB image just exceeds L2: DRAM reads 136 -> 75 MB per sweep, 43.9 -> 41.7 us).  The
-// order depends on the absolute sweep index, so split runs and resumes sum in the same order.
+// 134 MB image just exceeds L2: DRAM reads 136 -> 75 MB per sweep).  The order depends on the
+// absolute sweep index, so split runs and resumes sum in the same order.
 constexpr bool kRev = true;
-constexpr int kMaxStagesFp4 = 4;  // ring depth cap of the coupling-resident variant
-
-// Shared-memory plan of one kernel variant: NT output spins per CTA, operand variant OP.
-// The streamed variants fix the ring at compile time; the coupling-resident one sizes it at
-// run time around its resident coupling block (sweep_big_smem).
+// Shared-memory and tensor-memory plan of one kernel variant: NT output spins per CTA, operand
+// variant OP.
 template <int NT, int OP>
 struct BigCfg {
   static constexpr bool kReal = OP == kBigBf16, kFp4 = OP == kBigFp4;
   static constexpr int kSpinsPerKB = kFp4 ? 256 : (kReal ? 64 : 128);  // per 128-byte row
+  static constexpr int kWPK = kSpinsPerKB / 32;  // words of the bit image per row and K-block
   static constexpr int kSPT = NT / 4;            // spins per epilogue thread
   static constexpr int kChunks = kSPT / 16;      // 16-spin chunks per thread
-  static constexpr int kABytes = 128 * 128;      // one K-block of the spin tile (128 rows x 128 B)
   static constexpr int kBBytes = kFp4 ? 0 : NT * 128;  // streamed coupling rows per K-block
-  // K-blocks per ring stage: the coupling-resident variant streams only spins and copies
-  // three K-blocks (48 KB) at a time (SK N = 4096, two stages: 8.84 -> 8.45 us per sweep
-  // against two K-blocks through three stages; N = 2048: -2 %; N = 1024, 3072: equal).
-  static constexpr int kKPS = kFp4 ? 3 : KPS;
-  static constexpr int kAux = kReal ? 4096 * 4 : kTabWords * 4;  // noise levels | step table
-  static constexpr int kMisc = 4 * 128 * 4 + NT * 4 + 256;      // sRed, sH, barriers, flags
-  static constexpr int kFixed = 1024 + kAux + kMisc;
-  static constexpr int kFit = (kSmemBudget - kFixed) / (kKPS * (kABytes + kBBytes));
-  static constexpr int kStages = kFp4 ? kMaxStagesFp4 : (kFit < 8 ? kFit : 8);  // ring depth (max)
-  static constexpr int kSmem = kFixed + kStages * kKPS * (kABytes + kBBytes);
-  static constexpr int kTmemCols = kFp4 ? 2 * NT : NT;  // accumulator (+ unit scale factors)
-  static_assert(kFp4 || kFit >= 2, "ring too shallow");
+  static constexpr int kRing = kStages * kPB * kBBytes;
+  // Largest step table staged in shared memory (words): 8192, or what the ring leaves.
+  static constexpr int kTab = OP == kBigFp8 && NT == 128 ? 7680 : kTabWords;
+  static constexpr int kAux = kReal ? 4096 * 4 : kTab * 4;  // noise levels | step table
+  static constexpr int kMisc = 4 * 128 * 4 + NT * 4 + 256;  // sRed, sH, barriers, flags
+  static constexpr int kSmem = 1024 + kRing + kAux + kMisc;
+  static constexpr int kTmemA = kFp4 ? 2 * NT : NT;  // accumulator (+ unit scale factors), then A
+  static constexpr int kTmemCols = 512;
+  static_assert(kTmemA + kStages * kPB * kACols <= kTmemCols, "tensor memory");
+  static_assert(kFp4 || kSmem <= kSmemBudget, "shared memory");
   static_assert(!kFp4 || NT == 64, "the coupling-resident variant has 64-spin column blocks");
 };
 
-// Shared-memory plan of the coupling-resident variant for npad spins: [pad][ring][resident
-// couplings NT x npad / 2][table?][misc].  The 1024-byte alignment pad is reserved only when
-// it costs no ring stage; otherwise the kernel checks the base alignment itself.
+// Shared-memory plan of the coupling-resident variant for npad spins: [pad][resident couplings
+// NT x npad / 2][table?][misc].
 BigSmem fp4_plan(int npad, int stride_words) {
   using C = BigCfg<64, kBigFp4>;
   BigSmem out;
   if (npad % 256 != 0 || npad > 4096) return out;
-  const int stage = C::kKPS * C::kABytes;
-  const int jres = 64 * npad / 2;
-  const int avail = kSmemBudget - jres - C::kMisc;
-  auto fit = [&](int extra) { return (avail - extra) / stage; };
-  const int base = std::min(kMaxStagesFp4, fit(0));
-  const int pad = std::min(kMaxStagesFp4, fit(1024)) == base ? 1024 : 0;
-  // the step table goes to shared memory when the ring keeps at least 96 KB in flight beside it
-  const bool tab = stride_words <= kTabWords &&
-                   std::min(kMaxStagesFp4, fit(pad + kTabWords * 4)) * stage >= 3 * 32768;
-  out.stages = std::min(kMaxStagesFp4, fit(pad + (tab ? kTabWords * 4 : 0)));
-  out.tab_smem = tab ? 1 : 0;
-  out.bytes = pad + out.stages * stage + jres + (tab ? kTabWords * 4 : 0) + C::kMisc;
-  out.ok = out.stages >= 2 && out.bytes <= kSmemBudget;
+  out.tab_smem = stride_words <= C::kTab ? 1 : 0;
+  out.bytes = 1024 + 64 * npad / 2 + (out.tab_smem ? C::kTab * 4 : 0) + C::kMisc;
+  out.ok = out.bytes <= kSmemBudget;
   return out;
 }
 
-__device__ __forceinline__ void fence_proxy_async_global() {
-  asm volatile("fence.proxy.async.global;" ::: "memory");
+// ---- spins as bits: the image of one replica tile is [npad / 32 words][128 rows], each 16-bit half
+// holding 16 consecutive spins in the order its operand type expands with a shift and a mask:
+//   BF16  bit k = spin 2 k, bit 8 + k = spin 2 k + 1     (a register = spins 2 k, 2 k + 1)
+//   FP8   bit 4 b + j = spin 4 j + b                      (register j = spins 4 j .. 4 j + 3)
+//   E2M1  bits 4 m + 2 j, 4 m + 2 j + 1 = spins 8 j + 2 m, 8 j + 2 m + 1   (register j = spins 8 j ..
+//         8 j + 7; a pair of bits selects a byte of two nibbles)
+template <int OP>
+__device__ __forceinline__ uint32_t pack_spins16(uint32_t x) {
+  uint32_t t;
+  if constexpr (OP == kBigBf16) {
+    t = (x ^ (x >> 1)) & 0x2222u, x ^= t ^ (t << 1);
+    t = (x ^ (x >> 2)) & 0x0C0Cu, x ^= t ^ (t << 2);
+    t = (x ^ (x >> 4)) & 0x00F0u, x ^= t ^ (t << 4);
+  } else if constexpr (OP == kBigFp8) {
+    t = (x ^ (x >> 3)) & 0x0A0Au, x ^= t ^ (t << 3);
+    t = (x ^ (x >> 6)) & 0x00CCu, x ^= t ^ (t << 6);
+  } else {
+    t = (x ^ (x >> 4)) & 0x00F0u, x ^= t ^ (t << 4);
+    t = (x ^ (x >> 2)) & 0x0C0Cu, x ^= t ^ (t << 2);
+  }
+  return x;
+}
+
+// Half h of word w -> its operand registers v[0 .. kRegs - 1] (8 BF16, 4 FP8 or 2 E2M1).
+template <int OP>
+__device__ __forceinline__ void expand_spins16(uint32_t w, int h, uint32_t* v) {
+  if constexpr (OP == kBigBf16) {
+    const uint32_t z = __byte_perm(w, 0, h ? 0x3424 : 0x1404);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = ((z << (7 - k)) & 0x80008000u) ^ 0xBF80BF80u;
+  } else if constexpr (OP == kBigFp8) {
+    uint32_t z = __byte_perm(w, 0, h ? 0x4342 : 0x4140);
+    z = (z | (z << 4)) & 0x0F0F0F0Fu;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = ((z << (7 - j)) & 0x80808080u) ^ 0xB8B8B8B8u;
+  } else {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) v[j] = __byte_perm(0x222AA2AAu, 0, (w >> (16 * h + 2 * j)) & 0x3333u);
+  }
 }
 
 // Grid-wide barrier with a time bound over a monotone 64-bit arrival counter (bar[0..1],
@@ -124,11 +155,12 @@ __device__ __forceinline__ void grid_abort(unsigned int* bar) {
   atomicOr(reinterpret_cast<unsigned long long*>(bar), kBarAbort);
 }
 
+// Called by the epilogue threads; their first one arrives for the CTA.
 __device__ bool grid_barrier(unsigned int* bar, unsigned long long target, int* err, int* sflag,
                              uint64_t limit_ns) {
   const uint64_t limit = limit_ns ? limit_ns : 2000000000ull;
-  __syncthreads();
-  if (threadIdx.x == 0) {
+  asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory");
+  if (threadIdx.x == 64) {
     unsigned long long* cnt = reinterpret_cast<unsigned long long*>(bar);
     unsigned long long v;
     asm volatile("atom.add.acq_rel.gpu.global.u64 %0, [%1], 1;" : "=l"(v) : "l"(cnt) : "memory");
@@ -147,7 +179,7 @@ __device__ bool grid_barrier(unsigned int* bar, unsigned long long target, int* 
     }
     *sflag = (v & kBarAbort) ? 0 : 1;
   }
-  __syncthreads();
+  asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory");
   return *sflag != 0;
 }
 
@@ -156,38 +188,23 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_big_kernel(const __grid_con
   using C = BigCfg<NT, OP>;
   constexpr bool REAL = C::kReal, FP4 = C::kFp4;
   using EAcc = std::conditional_t<REAL, float, int>;  // energy partial sums
-  constexpr int kABytes = C::kABytes, kBBytes = C::kBBytes;
-  constexpr int kSPT = C::kSPT, kChunks = C::kChunks;
-  constexpr int kKPS = C::kKPS;
-  constexpr int kMaxStages = C::kStages;
-  const int kStages = FP4 ? L.stages : C::kStages;  // ring depth of this launch
+  constexpr int kBBytes = C::kBBytes;
+  constexpr int kSPT = C::kSPT, kChunks = C::kChunks, kWPK = C::kWPK;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  uint8_t* sA = smem;                               // kStages x kKPS x kABytes
-  uint8_t* sB = sA + kStages * kKPS * kABytes;      // kStages x kKPS x kBBytes (streamed)
-  uint8_t* sJ = sB + kStages * kKPS * kBBytes;      // resident couplings (FP4): NT x npad / 2
+  uint8_t* sB = smem;                               // kStages x kPB x kBBytes (streamed couplings)
+  uint8_t* sJ = sB + C::kRing;                      // resident couplings (FP4): NT x npad / 2
   const int jres_bytes = FP4 ? NT * L.P.npad / 2 : 0;
   const bool tab_smem = L.tab_smem != 0;
-  uint32_t* sTab = reinterpret_cast<uint32_t*>(sJ + jres_bytes);  // [kTabWords]
+  uint32_t* sTab = reinterpret_cast<uint32_t*>(sJ + jres_bytes);  // [C::kTab]
   float* sZ = reinterpret_cast<float*>(sTab);       // [4096] noise levels (real)
   const int aux_bytes = REAL ? C::kAux : (FP4 && !tab_smem ? 0 : C::kAux);
   EAcc* sRed = reinterpret_cast<EAcc*>(sJ + jres_bytes + aux_bytes);  // [4][128 rows]
   uint32_t* sH = reinterpret_cast<uint32_t*>(sRed + 4 * 128);  // [NT] bias: int32 or float bits
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sH + NT);       // full[S], empty[S], done, jres
-  uint32_t* sTmem = reinterpret_cast<uint32_t*>(bars + 2 * kMaxStages + 2);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sH + NT);
+  uint32_t* sTmem = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 3);
   int* sFlag = reinterpret_cast<int*>(sTmem + 1);
-  if constexpr (FP4) {
-    // The plan may leave no room for the alignment pad: check that the layout fits what the
-    // launch provided (uniform over the grid, so every CTA returns before any barrier).
-    uint32_t dyn;
-    asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
-    const uint32_t end = static_cast<uint32_t>(reinterpret_cast<uint8_t*>(sFlag + 1) - smem_raw);
-    if (end > dyn) {
-      if (threadIdx.x == 0) atomicOr(L.err, kDevErrLayout);
-      return;
-    }
-  }
 
   const Problem& P = L.P;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -211,10 +228,11 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_big_kernel(const __grid_con
   const uint32_t full_mask = kSPT == 32 ? 0xFFFFFFFFu : ((1u << (kSPT & 31)) - 1u);
   const uint32_t vmask = valid >= kSPT ? full_mask : (valid > 0 ? (1u << valid) - 1u : 0u);
 
-  const uint32_t bar_full0 = smem_u32(&bars[0]);
-  const uint32_t bar_empty0 = smem_u32(&bars[kMaxStages]);
-  const uint32_t bar_done = smem_u32(&bars[2 * kMaxStages]);
-  const uint32_t bar_jres = smem_u32(&bars[2 * kMaxStages + 1]);
+  const uint32_t bar_full0 = smem_u32(&bars[0]);          // a stage's spins and couplings
+  const uint32_t bar_empty0 = smem_u32(&bars[kStages]);
+  const uint32_t bar_done = smem_u32(&bars[2 * kStages]);  // a sweep's MMAs
+  const uint32_t bar_jres = bar_done + 8;                          // resident couplings
+  const uint32_t bar_tab = bar_done + 16;                          // the step's table
 
   if (warp == 1) {
     tmem_alloc(smem_u32(sTmem), C::kTmemCols);
@@ -222,11 +240,12 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_big_kernel(const __grid_con
   }
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
-      mbar_init(bar_full0 + 8 * s, 1);
+      mbar_init(bar_full0 + 8 * s, kEpiWarps + (FP4 ? 0 : 1));
       mbar_init(bar_empty0 + 8 * s, 1);
     }
     mbar_init(bar_done, 1);
     mbar_init(bar_jres, 1);
+    mbar_init(bar_tab, 1);
     fence_mbar_init();
   }
   for (int k = tid; k < NT; k += kThreads) {
@@ -291,137 +310,153 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_big_kernel(const __grid_con
   if (!L.cont) best = cur;
   const bool has_target = P.has_target != 0;
 
-  // Spin image s(t) for this CTA's block (rows of the tile, its NT spins): FP8, BF16 or E2M1
-  // +-1.  The image is tile-major, [replica tile][K-block][128 rows x 128 B with the 128-byte
-  // swizzle], so consecutive K-blocks of one tile are contiguous (one copy per ring stage).
-  const size_t tile_bytes = static_cast<size_t>(kblocks) * kABytes;
-  auto write_image = [&](uint8_t* img, uint32_t bits) {
-    if (!epi || col0 >= npad) return;
-    uint8_t* base = img + static_cast<size_t>(rt) * tile_bytes;
-#pragma unroll
-    for (int c = 0; c < kChunks; ++c) {
-      const uint32_t b16 = (bits >> (16 * c)) & 0xFFFFu;
-      const int k = col0 + 16 * c;
-      if constexpr (REAL) {
-        *reinterpret_cast<uint4*>(base + sw128_offset(row, 2 * k, 128)) = bf16x8_from_bits(b16 & 0xFFu);
-        *reinterpret_cast<uint4*>(base + sw128_offset(row, 2 * k + 16, 128)) = bf16x8_from_bits(b16 >> 8);
-      } else if constexpr (FP4) {
-        // 16 spins = 8 bytes at byte k / 2 of the row (k is a multiple of 16).
-        *reinterpret_cast<uint2*>(base + sw128_offset(row, k >> 1, 128)) =
-            make_uint2(e2m1x8_from_bits(b16 & 0xFFu), e2m1x8_from_bits(b16 >> 8));
-      } else {
-        *reinterpret_cast<uint4*>(base + sw128_offset(row, k, 128)) = fp8x16_from_bits(b16);
-      }
-    }
+  // Bit image of s(t): this thread's spins (the rows of the tile, the CTA's NT spins).
+  const size_t tile_words = static_cast<size_t>(npad / 32) * 128;
+  auto write_image = [&](uint32_t* img, uint32_t bits) {
+    if (!epi) return;
+    uint32_t* word = img + rt * tile_words + static_cast<size_t>(col0 >> 5) * 128 + row;
+    if constexpr (kSPT == 32)
+      *word = pack_spins16<OP>(bits & 0xFFFFu) | (pack_spins16<OP>(bits >> 16) << 16);
+    else
+      reinterpret_cast<uint16_t*>(word)[(col0 >> 4) & 1] = static_cast<uint16_t>(pack_spins16<OP>(bits));
   };
-  unsigned long long bar_target = nblocks;  // counter value that completes the next barrier
-  write_image(L.s_img[0], cur & vmask);
-  fence_proxy_async_global();
-  if (!grid_barrier(L.bar, bar_target, L.err, sFlag, L.wait_ns)) goto teardown;
+  bool aborted = false;  // on every thread of the role that gave up
 
   {
-    // ring positions: stage and phase of the next load (the first round waits for nothing) / MMA
-    uint32_t ld_stage = 0, ld_phase = 0xFFFFFFFFu, mma_stage = 0, mma_phase = 0, done_phase = 0;
     const uint32_t idesc = REAL ? idesc_bf16(128, NT) : (FP4 ? idesc_mxf4(128, NT) : idesc_e4m3(128, NT));
-    bool jres_ready = !FP4;
-    // Producer (warp 0, converged, one elected lane): stream the K blocks of image `img` (spins of the tile) and, unless
-    // they are resident, of the coupling rows of the column block into the ring.  A stage
-    // is refilled once the MMAs that read it have completed (its empty barrier).
-    // A stage holds kKPS consecutive K-blocks: the tile's spins of all of them in one copy
-    // (the image is tile-major), streamed coupling rows in one copy per K-block.
-    auto produce = [&](const uint8_t* img, bool rev) -> bool {
-      const uint8_t* a_src = img + static_cast<size_t>(rt) * tile_bytes;
+    const int nst = (kblocks + kPB - 1) / kPB;  // ring stages of a sweep
+    // Stages used so far, the same count in every role: stage g lies in slot g % kStages.
+    uint32_t gs = 0;
+    // K-block at position p of a sweep: in order, or pair by pair from the end
+    auto kb_at = [&](int p, bool rev) {
+      if (!rev) return p;
+      const int pairs = (kblocks + KPS - 1) / KPS, first = kblocks - (pairs - 1) * KPS;
+      return p < first ? (pairs - 1) * KPS + p : (pairs - 2 - (p - first) / KPS) * KPS + (p - first) % KPS;
+    };
+    // Whether slot of stage g may be filled (bounded wait for the MMAs of its last use).
+    auto slot_free = [&](uint32_t g) -> bool {
+      return __all_sync(0xFFFFFFFFu, g < kStages || mbar_wait_fast(bar_empty0 + 8 * (g % kStages),
+                                                                   (g / kStages - 1) & 1, L.wait_ns));
+    };
+    // Producer (warp 0, converged, one elected lane): the coupling rows of the column block.  They
+    // do not depend on the spins, so it runs ahead into the next sweep as slots become free.
+    auto produce = [&](bool rev) -> bool {
       // Coupling images of n > 256 are chunk-major: 16 KB blocks of 128 rows x one K-block,
-      // ordered [row block][K-block], so the stage's K-blocks of a 128-row column block are
+      // ordered [row block][K-block], so consecutive K-blocks of a 128-row column block are
       // one copy; a 64-row column block is half of each 16 KB block (one copy per K-block).
       const uint8_t* b_src = P.jimg + static_cast<size_t>(NT == 128 ? cb : cb >> 1) * kblocks * 16384 +
                              (NT == 128 ? 0 : (cb & 1) * 8192);
-      const int nst = (kblocks + kKPS - 1) / kKPS;
-      for (int si = 0; si < nst; ++si) {
-        const int kb0 = (rev ? nst - 1 - si : si) * kKPS;
-        const int nk = kblocks - kb0 < kKPS ? kblocks - kb0 : kKPS;
-        const uint32_t s = ld_stage;
-        if (!__all_sync(0xFFFFFFFFu, ld_phase == 0xFFFFFFFFu ||
-                                         mbar_wait_fast(bar_empty0 + 8 * s, ld_phase & 1, L.wait_ns)))
-          return false;
+      for (int si = 0; si < nst; ++si, ++gs) {
+        const int p0 = si * kPB, nk = kblocks - p0 < kPB ? kblocks - p0 : kPB;
+        if (!slot_free(gs)) return false;
+        const uint32_t slot = gs % kStages;
         if (elect_one()) {
-          mbar_expect_tx(bar_full0 + 8 * s, nk * (kABytes + kBBytes));
-          bulk_g2s(smem_u32(sA) + s * kKPS * kABytes, a_src + static_cast<size_t>(kb0) * kABytes,
-                   nk * kABytes, bar_full0 + 8 * s);
-          if constexpr (kBBytes > 0) {
-            if constexpr (NT == 128) {
-              bulk_g2s(smem_u32(sB) + s * kKPS * kBBytes, b_src + static_cast<size_t>(kb0) * 16384,
-                       nk * kBBytes, bar_full0 + 8 * s);
-            } else {
-#pragma unroll
-              for (int j = 0; j < kKPS; ++j)
-                if (j < nk)
-                  bulk_g2s(smem_u32(sB) + (s * kKPS + j) * kBBytes,
-                           b_src + static_cast<size_t>(kb0 + j) * 16384, kBBytes, bar_full0 + 8 * s);
-            }
+          const uint32_t full = bar_full0 + 8 * slot;
+          mbar_expect_tx(full, nk * kBBytes);
+          for (int j = 0; j < nk;) {
+            const int kb = kb_at(p0 + j, rev);
+            int run = 1;
+            if (NT == 128)
+              while (j + run < nk && kb_at(p0 + j + run, rev) == kb + run) ++run;
+            bulk_g2s(smem_u32(sB) + (slot * kPB + j) * kBBytes, b_src + static_cast<size_t>(kb) * 16384,
+                     run * kBBytes, full);
+            j += run;
           }
         }
         __syncwarp();
-        if (++ld_stage == static_cast<uint32_t>(kStages)) {
-          ld_stage = 0;
-          ++ld_phase;
-        }
       }
       return true;
     };
-    // MMA issuer (warp 1, converged, one elected lane): D = S_tile x J_block^T, K block by K
-    // block as stages land; it never waits for an MMA to finish, only for data.  Each MMA
+    // Epilogue warps: the tile's spins from the bit image into tensor memory, K-block `grp` of
+    // every stage into this warp's lane quadrant.  The next stage's words are in flight meanwhile (more
+    // stages ahead, 2 to 8, measured the same or slower).
+    auto expand = [&](const uint32_t* img, bool rev) -> bool {
+      const uint32_t* src = img + rt * tile_words + row;
+      uint32_t w[kWPK];
+      auto fetch = [&](int p) {
+        if (p >= kblocks) return;
+        const uint32_t* at = src + static_cast<size_t>(kb_at(p, rev)) * kWPK * 128;
+#pragma unroll
+        for (int k = 0; k < kWPK; ++k) w[k] = __ldcg(at + k * 128);
+      };
+      fetch(grp);
+      for (int p = grp; p - grp < kblocks; p += kPB, ++gs) {
+        if (!slot_free(gs)) return false;
+        tc_fence_after();
+        const uint32_t slot = gs % kStages;
+        if (p < kblocks) {
+          const uint32_t ta = tmem + (static_cast<uint32_t>(quad * 32) << 16) + C::kTmemA +
+                              (slot * kPB + grp) * kACols;
+          constexpr int kRegs = 16 / kWPK;  // operand registers of a 16-spin half
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            uint32_t v[16];
+#pragma unroll
+            for (int k = 0; k < kWPK; ++k) {
+              const int hw = i * kWPK + k;  // half word of the K-block
+              expand_spins16<OP>(w[hw >> 1], hw & 1, v + k * kRegs);
+            }
+            tmem_st16(ta + 16 * i, v);
+          }
+          fetch(p + kPB);
+          tmem_wait_st();
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_full0 + 8 * slot);
+      }
+      return true;
+    };
+    // MMA issuer (warp 1, converged, one elected lane): D = S_tile x J_block^T, stage by stage as
+    // spins and couplings land; it never waits for an MMA to finish, only for data.  Each MMA
     // consumes 32 bytes of K (32 FP8, 16 BF16 or 64 E2M1 values).
     auto multiply = [&](bool rev) -> bool {
-      if (!jres_ready) {
-        if (!__all_sync(0xFFFFFFFFu, mbar_wait_fast(bar_jres, 0, L.wait_ns))) return false;
-        jres_ready = true;
-      }
-      const uint64_t a_desc = sw128_desc(smem_u32(sA)), b_desc = sw128_desc(smem_u32(FP4 ? sJ : sB));
-      const int nst = (kblocks + kKPS - 1) / kKPS;
-      for (int si = 0; si < nst; ++si) {
-        const int kb0 = (rev ? nst - 1 - si : si) * kKPS;
-        const int nk = kblocks - kb0 < kKPS ? kblocks - kb0 : kKPS;
-        const uint32_t s = mma_stage;
-        if (!__all_sync(0xFFFFFFFFu, mbar_wait_fast(bar_full0 + 8 * s, mma_phase & 1, L.wait_ns))) return false;
+      const uint64_t b_desc = sw128_desc(smem_u32(FP4 ? sJ : sB));
+      for (int si = 0; si < nst; ++si, ++gs) {
+        const int p0 = si * kPB, nk = kblocks - p0 < kPB ? kblocks - p0 : kPB;
+        const uint32_t slot = gs % kStages;
+        if (!__all_sync(0xFFFFFFFFu, mbar_wait_fast(bar_full0 + 8 * slot, (gs / kStages) & 1, L.wait_ns)))
+          return false;
         tc_fence_after();
         if (elect_one()) {
-          const uint64_t a0 = a_desc + s * (kKPS * kABytes >> 4);
-          const uint64_t b0 = b_desc + (FP4 ? kb0 * (NT * 128 >> 4) : s * (kKPS * kBBytes >> 4));
+          const uint32_t a0 = tmem + C::kTmemA + slot * kPB * kACols;
 #pragma unroll
-          for (int j = 0; j < kKPS; ++j)
+          for (int j = 0; j < kPB; ++j)
             if (j < nk) {
+              const uint64_t bj = b_desc + (FP4 ? kb_at(p0 + j, rev) * (NT * 128 >> 4)
+                                                : (slot * kPB + j) * (kBBytes >> 4));
 #pragma unroll
               for (int ks = 0; ks < 4; ++ks) {
                 const uint32_t acc = (si > 0 || j > 0 || ks > 0) ? 1u : 0u;
-                const uint64_t a = a0 + j * (kABytes >> 4) + 2 * ks;
-                const uint64_t b = b0 + j * ((FP4 ? NT * 128 : kBBytes) >> 4) + 2 * ks;
                 if constexpr (REAL)
-                  mma_bf16(tmem, a, b, idesc, acc);
+                  mma_bf16_ta(tmem, a0 + j * kACols + 8 * ks, bj + 2 * ks, idesc, acc);
                 else if constexpr (FP4)
-                  mma_mxf4(tmem, a, b, idesc, tmem + NT, tmem + NT, acc);
+                  mma_mxf4_ta(tmem, a0 + j * kACols + 8 * ks, bj + 2 * ks, idesc, tmem + NT, tmem + NT, acc);
                 else
-                  mma_e4m3(tmem, a, b, idesc, acc);
+                  mma_f8_ta(tmem, a0 + j * kACols + 8 * ks, bj + 2 * ks, idesc, acc);
               }
             }
-          mma_commit(bar_empty0 + 8 * s);
           if (si + 1 == nst) mma_commit(bar_done);
+          mma_commit(bar_empty0 + 8 * slot);
         }
         __syncwarp();
-        if (++mma_stage == static_cast<uint32_t>(kStages)) {
-          mma_stage = 0;
-          ++mma_phase;
-        }
       }
       return true;
+    };
+    auto give_up = [&]() {
+      aborted = true;
+      if (lane == 0) {
+        atomicOr(L.err, kDevErrTimeout);
+        grid_abort(L.bar);
+      }
     };
 
     // Best / first-hit bookkeeping of state `state` = s(tt) from its replica energy, complete
     // since the barrier that ended sweep tt.  Returns that energy.
     EAcc* energy = reinterpret_cast<EAcc*>(L.energy);
-    auto track = [&](int tt, uint32_t state) -> EAcc {
-      // L2 read: the accumulator was written by other SMs during sweep tt.
-      const EAcc etot = __ldcg(&energy[((tt - t_begin) % 3) * rpad + rl]);
+    // L2 read: the accumulator was written by other SMs during sweep tt.
+    auto summed = [&](int tt) { return __ldcg(&energy[((tt - t_begin) % 3) * rpad + rl]); };
+    auto track = [&](int tt, uint32_t state, EAcc etot) -> EAcc {
       EAcc E;
       bool hit;
       if constexpr (REAL) {
@@ -440,40 +475,45 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_big_kernel(const __grid_con
       return E;
     };
 
+    if (warp == 0) {
+      if constexpr (!FP4)
+        for (int t = t_begin; t <= t_end; ++t) {
+          // Injected fault: nothing is loaded in the first sweep, so the MMA warp's first
+          // wait cannot complete.
+          if (L.inject == 1 && t == t_begin) break;
+          if (!produce(kRev && (t & 1))) {
+            give_up();
+            break;
+          }
+        }
+    } else if (warp == 1) {
+      bool ok = !FP4 || __all_sync(0xFFFFFFFFu, mbar_wait_fast(bar_jres, 0, L.wait_ns));
+      for (int t = t_begin; t <= t_end && ok; ++t) ok = multiply(kRev && (t & 1));
+      if (!ok) give_up();
+    } else {  // ---- epilogue warps
+    unsigned long long bar_target = nblocks;  // counter value that completes the next barrier
+    write_image(reinterpret_cast<uint32_t*>(L.s_img[0]), cur & vmask);
+    aborted = !grid_barrier(L.bar, bar_target, L.err, sFlag, L.wait_ns);
     int cur_img = 0;
+    uint32_t done_phase = 0;
     uint32_t prev = 0;  // s(t-1) of this thread's spins, until its energy has been tracked
-    for (int t = t_begin; t <= t_end; ++t) {
+    for (int t = t_begin; t <= t_end && !aborted; ++t) {
       const bool last = t == t_end;
-      if (warp == 0) {
-        fence_proxy_async_global();
-        // Injected fault: nothing is loaded in the first sweep, so the MMA thread's first
-        // wait cannot complete.
-        if (!(L.inject == 1 && t == t_begin) && !produce(L.s_img[cur_img], kRev && (t & 1)) && lane == 0) {
-          atomicOr(L.err, kDevErrTimeout);
-          grid_abort(L.bar);
-        }
-      } else if (warp == 1) {
-        if (!multiply(kRev && (t & 1)) && lane == 0) {
-          atomicOr(L.err, kDevErrTimeout);
-          grid_abort(L.bar);
-        }
+      // The step's table (the last step's reads ended before the grid barrier).
+      if (!REAL && tab_smem && !last && tid == 64) {
+        mbar_expect_tx(bar_tab, P.stride_words * 4);
+        bulk_g2s(smem_u32(sTab), P.thr + static_cast<size_t>(t) * P.stride_words, P.stride_words * 4, bar_tab);
       }
       // Zero the energy buffer that sweep t+1 will accumulate into (see header).
-      if (cb == 0 && epi && grp == 0) __stcg(&energy[((t - t_begin + 1) % 3) * rpad + rl], EAcc(0));
+      if (cb == 0 && grp == 0) __stcg(&energy[((t - t_begin + 1) % 3) * rpad + rl], EAcc(0));
       EAcc eacc = 0;
       uint32_t nxt = 0;
-      if (epi) {
-        // While the MMAs run: the bookkeeping of s(t-1), whose energy the last barrier
-        // completed, and this step's thresholds staged (the previous step's reads ended
-        // before that barrier); then sync the 16 epilogue warps.
-        if (t > t_begin) track(t - 1, prev);
-        if (!REAL && tab_smem && !last) {
-          const uint4* src =
-              reinterpret_cast<const uint4*>(P.thr + static_cast<size_t>(t) * P.stride_words);
-          for (int k = tid - 64; k < P.stride_words / 4; k += kEpiWarps * 32)
-            reinterpret_cast<uint4*>(sTab)[k] = __ldg(src + k);
-        }
-        asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory");
+      {
+        const EAcc etot = t > t_begin ? summed(t - 1) : EAcc(0);
+        bool ok = (L.inject == 1 && t == t_begin) || expand(reinterpret_cast<const uint32_t*>(L.s_img[cur_img]), kRev && (t & 1));
+        // While the last MMAs run: the bookkeeping of s(t-1), whose energy the last barrier
+        // completed.
+        if (t > t_begin) track(t - 1, prev, etot);
         // The sweep's noise while the MMAs run: draws (integer couplings) or xi s + eta z (real).
         uint32_t rw[kSPT / 2];
         float ns[REAL ? kSPT : 1];
@@ -497,10 +537,12 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_big_kernel(const __grid_con
               ns[e] = __fmaf_rn(eta, sZ[key], ((cur >> e) & 1u) ? P.xi : -P.xi);
             }
         }
-        const bool ok = __all_sync(0xFFFFFFFFu, mbar_wait_fast(bar_done, done_phase, L.wait_ns));
+        ok = __all_sync(0xFFFFFFFFu, ok && mbar_wait_fast(bar_done, done_phase, L.wait_ns) &&
+                                         (REAL || !tab_smem || last ||
+                                          mbar_wait_fast(bar_tab, static_cast<uint32_t>(t - t_begin) & 1, L.wait_ns)));
         if (!ok && lane == 0) {
           atomicOr(L.err, kDevErrTimeout);
-          grid_abort(L.bar);
+          grid_abort(L.bar);  // the grid barrier below returns false on every thread
         }
         tc_fence_after();
         if (warp_active && ok) {
@@ -593,51 +635,50 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_big_kernel(const __grid_con
         sRed[grp * 128 + row] = eacc;
       }
       done_phase ^= 1;
-      if (!last) write_image(L.s_img[cur_img ^ 1], nxt);
+      if (!last) write_image(reinterpret_cast<uint32_t*>(L.s_img[cur_img ^ 1]), nxt);
       tc_fence_before();
-      __syncthreads();
-      if (epi && grp == 0) {
+      asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory");
+      if (grp == 0) {
         const EAcc tot = sRed[row] + sRed[128 + row] + sRed[256 + row] + sRed[384 + row];
         atomicAdd(&energy[((t - t_begin) % 3) * rpad + rl], tot);
       }
-      fence_proxy_async_global();
       bar_target += nblocks;
-      if (!grid_barrier(L.bar, bar_target, L.err, sFlag, L.wait_ns)) goto teardown;
-      if (epi) {
-        if (last) {
-          const EAcc E = track(t, cur);
-          if (row_valid) {
+      aborted = !grid_barrier(L.bar, bar_target, L.err, sFlag, L.wait_ns);
+      if (aborted) break;
+      if (last) {
+        const EAcc E = track(t, cur, summed(t));
+        if (row_valid) {
 #pragma unroll
-            for (int c = 0; c < kChunks; ++c)
-              if (chunk + c < half_words) {
-                const size_t o = static_cast<size_t>(r) * half_words + chunk + c;
-                reinterpret_cast<uint16_t*>(P.cur_bits)[o] = static_cast<uint16_t>(cur >> (16 * c));
-                reinterpret_cast<uint16_t*>(P.best_bits)[o] = static_cast<uint16_t>(best >> (16 * c));
-              }
-            if (cb == 0 && grp == 0) {
-              P.best_E[r] = static_cast<double>(best_E);
-              P.best_t[r] = best_t;
-              P.first_hit[r] = first_hit;
-              P.final_E[r] = static_cast<double>(E);
+          for (int c = 0; c < kChunks; ++c)
+            if (chunk + c < half_words) {
+              const size_t o = static_cast<size_t>(r) * half_words + chunk + c;
+              reinterpret_cast<uint16_t*>(P.cur_bits)[o] = static_cast<uint16_t>(cur >> (16 * c));
+              reinterpret_cast<uint16_t*>(P.best_bits)[o] = static_cast<uint16_t>(best >> (16 * c));
             }
+          if (cb == 0 && grp == 0) {
+            P.best_E[r] = static_cast<double>(best_E);
+            P.best_t[r] = best_t;
+            P.first_hit[r] = first_hit;
+            P.final_E[r] = static_cast<double>(E);
           }
-        } else {
-          prev = cur;
-          cur = nxt;
         }
+      } else {
+        prev = cur;
+        cur = nxt;
       }
       cur_img ^= 1;
     }
+    }
   }
 
-teardown:
+  // A wait gave up: copies and MMAs in flight need microseconds; the other roles end on their own
+  // bounded waits.
+  if (aborted) __nanosleep(20000);
   tc_fence_before();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem, C::kTmemCols);
 }
 
-// Kernel and co-resident CTAs of the (NT, OP) variant at `smem` bytes of dynamic shared
-// memory (the attribute is set to the whole budget, so any plan of the variant launches).
 template <int NT, int OP>
 cudaError_t variant_setup(int smem, const void** fn, int* max_blocks) {
   *fn = reinterpret_cast<const void*>(sweep_big_kernel<NT, OP>);
@@ -671,8 +712,7 @@ template <int NT, int OP>
 BigSmem streamed_plan(int stride_words) {
   BigSmem out;
   out.ok = true;
-  out.stages = BigCfg<NT, OP>::kStages;
-  out.tab_smem = OP == kBigFp8 && stride_words <= kTabWords ? 1 : 0;
+  out.tab_smem = OP == kBigFp8 && stride_words <= BigCfg<NT, OP>::kTab ? 1 : 0;
   out.bytes = BigCfg<NT, OP>::kSmem;
   return out;
 }
@@ -701,7 +741,7 @@ int sweep_big_max_blocks(int nt, int op, int npad, int stride_words) {
 
 cudaError_t launch_sweep_big(const BigLaunch& L, int nt, int op, int blocks, cudaStream_t st) {
   const BigSmem plan = sweep_big_smem(nt, op, L.P.npad, L.P.stride_words);
-  if (!plan.ok || L.stages != plan.stages || L.tab_smem != plan.tab_smem) return cudaErrorInvalidValue;
+  if (!plan.ok || L.tab_smem != plan.tab_smem) return cudaErrorInvalidValue;
   if (op == kBigFp4 && L.j4 == nullptr) return cudaErrorInvalidValue;
   const void* fn = nullptr;
   int cap = 0;

@@ -71,17 +71,6 @@ __device__ __forceinline__ void put_spins32_tm(uint32_t tlane, int col, uint32_t
                : "memory");
 }
 
-// D (+)= A B with A (128 x 32 FP8, K-major) in tensor memory at a_tmem.
-__device__ __forceinline__ void mma_f8_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc,
-                                          uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
 constexpr float kMagic = 12582912.0f;      // 1.5 * 2^23: integer D in the low mantissa bits
 constexpr uint32_t kMagicBits = 0x4B400000u;
 

@@ -89,16 +89,15 @@ cudaError_t launch_serve_float(const Launch& L, const ServeQueue& Q, int nmax, i
 //             E2M1 for the whole launch and only E2M1 spins stream (integer couplings in
 //             {0, +-1, +-2, +-3, +-4, +-6}, npad <= 4096, nt = 64).
 enum BigOp : int { kBigFp8 = 0, kBigBf16 = 1, kBigFp4 = 2 };
-// Shared-memory plan of a variant: ring depth, whether the step's threshold table is staged
-// in shared memory, dynamic shared-memory bytes.  ok = false when the variant does not fit.
+// Shared-memory plan of a variant: whether the step's threshold table is staged in shared
+// memory, dynamic shared-memory bytes.  ok = false when the variant does not fit.
 struct BigSmem {
   bool ok = false;
-  int stages = 0;
   int tab_smem = 0;
   int bytes = 0;
 };
 BigSmem sweep_big_smem(int nt, int op, int npad, int stride_words);
-// L.stages / L.tab_smem must hold sweep_big_smem's plan for (nt, op, P.npad, P.stride_words).
+// L.tab_smem must hold sweep_big_smem's plan for (nt, op, P.npad, P.stride_words).
 cudaError_t launch_sweep_big(const BigLaunch& L, int nt, int op, int blocks, cudaStream_t st);
 // Co-resident CTAs on the current device for that plan (0 on error or when it does not fit).
 int sweep_big_max_blocks(int nt, int op, int npad, int stride_words);

@@ -10,8 +10,6 @@ enum : int {
   kDevErrTimeout = 1,      // a bounded mbarrier wait gave up
   kDevErrFieldRange = 2,   // a field fell outside the threshold table (cannot happen for
                            // a valid instance; checked so a bad table never reads out of range)
-  kDevErrLayout = 4,       // dynamic shared memory not 1024-byte aligned where the kernel's
-                           // layout has no room for the alignment pad (the kernel did nothing)
 };
 
 // Per-instance parameters of one launch.  All pointers are device pointers.
@@ -157,12 +155,9 @@ struct ServeQueue {
 // (replica tiles) x (nt-spin column blocks).
 struct BigLaunch {
   Problem P;
-  uint8_t* s_img[2];       // spin images (A operand), ping-pong: tile-major,
-                           // [rpad/128][K-blocks][128 rows x 128 B, 128-byte swizzle];
-                           // a 128-byte row holds 128 FP8, 64 BF16 or 256 E2M1 spins
+  uint8_t* s_img[2];       // spin images (bits), ping-pong: [rpad/128 tiles][npad/32 words][128 rows]
   const uint8_t* j4;       // E2M1 coupling image of the coupling-resident variant (else null)
-  int stages;              // K-block ring depth and threshold-table placement of the
-  int tab_smem;            //   variant's shared-memory plan
+  int tab_smem;            // the step's threshold table is staged in shared memory
   float* energy;           // [3][rpad] rotating per-replica energy accumulators (zeroed);
                            // int32 for integer couplings, float for real couplings
   int nt;                  // output spins per CTA (64 or 128)

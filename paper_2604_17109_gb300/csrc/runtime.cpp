@@ -1407,11 +1407,8 @@ int plan_big(int n, int npad, int R, bool real, bool fp4, int stride_words, BigP
 // Large-N anneal of one instance: the replicas are split into groups of tiles that fit the
 // co-resident grid (each group is an independent cooperative launch); per launch scratch
 // (two spin images, energy accumulators, barrier words) comes from the stream-ordered pool.
-// Bytes of one large-N spin image of rpad replica rows.
-size_t big_image_bytes(int rpad, int npad, int op) {
-  const size_t cells = static_cast<size_t>(rpad) * npad;
-  return op == kBigFp4 ? cells / 2 : (op == kBigBf16 ? 2 * cells : cells);
-}
+// Bytes of one large-N spin image (bits) of rpad replica rows.
+size_t big_image_bytes(int rpad, int npad) { return static_cast<size_t>(rpad) * npad / 8; }
 
 int launch_big(const Problem& P, bool real, int t_begin, int sweeps, uint64_t seed, bool cont,
                int* d_err, char* scratch, int* launches, cudaStream_t st) {
@@ -1425,7 +1422,7 @@ int launch_big(const Problem& P, bool real, int t_begin, int sweeps, uint64_t se
   for (int tile0 = 0; tile0 < tiles_total; tile0 += plan.tiles_per_launch) {
     const int tiles = std::min(plan.tiles_per_launch, tiles_total - tile0);
     const int rpad = tiles * 128;
-    const size_t img_bytes = big_image_bytes(rpad, P.npad, plan.op);
+    const size_t img_bytes = big_image_bytes(rpad, P.npad);
     const size_t energy_bytes = sizeof(float) * 3 * rpad;
     const size_t bytes = 2 * img_bytes + energy_bytes + 256;
     char* d = scratch;
@@ -1437,7 +1434,6 @@ int launch_big(const Problem& P, bool real, int t_begin, int sweeps, uint64_t se
     L.s_img[0] = reinterpret_cast<uint8_t*>(d);
     L.s_img[1] = reinterpret_cast<uint8_t*>(d + img_bytes);
     L.j4 = plan.op == kBigFp4 ? P.jimg4 : nullptr;
-    L.stages = smem.stages;
     L.tab_smem = smem.tab_smem;
     L.energy = reinterpret_cast<float*>(d + 2 * img_bytes);
     L.bar = reinterpret_cast<unsigned int*>(d + 2 * img_bytes + energy_bytes);
@@ -1798,7 +1794,7 @@ int build_plan(pim_instance* const* insts, int count, const int* replicas, const
       const int rc = plan_big(P.n, P.npad, P.R, insts[k]->real, P.jimg4 != nullptr, P.stride_words, &plan);
       if (rc != PIM_OK) return rc;
       const int rpad = plan.tiles_per_launch * 128;
-      B.big_scratch = std::max(B.big_scratch, 2 * big_image_bytes(rpad, P.npad, plan.op) +
+      B.big_scratch = std::max(B.big_scratch, 2 * big_image_bytes(rpad, P.npad) +
                                                   sizeof(float) * 3 * rpad + 256);
       continue;
     }
