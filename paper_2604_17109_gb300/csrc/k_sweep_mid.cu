@@ -37,7 +37,15 @@ constexpr int kMaxNpad = 1024;
 constexpr int kMaxChunks = kMaxNpad / kNT;
 constexpr int kStages = 3;                  // coupling ring depth
 constexpr int kBufs = 2;                    // TMEM accumulators of kNT columns
-constexpr int kTabWords = 4096;             // threshold table of one step in shared memory
+// Threshold table in shared memory.  A step's table of up to kTabHalf words (imax <= 1023, diagonal
+// encoding with dk <= 1024) lies in the half of its parity: the MMA warp has copied it
+// while the sweep before was decided, and no thread waits at the start of a sweep.  A larger table
+// takes both halves and is loaded by the epilogue threads between two barriers; past kTabWords it is
+// read from global memory.  Loading every table between barriers cost 460 - 1800 of a sweep's 15.7 k
+// (N = 512) to 33 k (N = 1000) cycles: SK N = 512 x 152 15.6 -> 14.9 us per sweep, N = 1000 x 152
+// 35.2 -> 32.8.
+constexpr int kTabWords = 4096;
+constexpr int kTabHalf = kTabWords / 2;
 constexpr int kEpiWarps = 16;
 constexpr int kGroups = kEpiWarps / 4;      // column groups per chunk
 constexpr int kCols = kNT / kGroups;        // columns of a chunk per epilogue thread
@@ -52,7 +60,7 @@ constexpr int kBlockBytes = kNT * 128;      // one K-block of 128 coupling rows
 // stages beat 2 x 6, 3 x 4 and 6 x 2 on the uneven batch).
 constexpr int kKPS = 4;
 constexpr int kStageBytes = kKPS * kBlockBytes;
-constexpr int kBarCount = 2 * kStages + 2 * kBufs + 2;
+constexpr int kBarCount = 2 * kStages + 2 * kBufs + 4;
 
 // Bounded wait with the common case (phase already complete) inline; the out-of-line wait
 // sleeps inside try_wait between checks.
@@ -222,8 +230,8 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   uint8_t* sRing = smem;
   uint32_t* sTab = reinterpret_cast<uint32_t*>(sRing + kStages * kStageBytes);
-  int* sRed = reinterpret_cast<int*>(sTab + kTabWords);  // [kGroups][128 rows]
-  int* sH = sRed + kGroups * 128;                         // [kMaxNpad]
+  int* sRed = reinterpret_cast<int*>(sTab + kTabWords);  // [2][kGroups][128 rows]
+  int* sH = sRed + 2 * kGroups * 128;                     // [kMaxNpad]
   uint64_t* bars = reinterpret_cast<uint64_t*>(sH + kMaxNpad);
   uint32_t* sTmem = reinterpret_cast<uint32_t*>(bars + kBarCount);
   volatile int* sUnit = reinterpret_cast<volatile int*>(sTmem + 1);
@@ -232,7 +240,10 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool epi = warp >= 2;
   const int quad = warp & 3;                    // TMEM lane quadrant of this warp
-  const int grp = epi ? (warp - 2) >> 2 : 0;    // group of kCols columns inside a chunk
+  // Group of kCols columns inside a chunk.  The shuffles here and for P.q tell the compiler that the
+  // value is the same on every lane: what the noise blocks need of it then lives in uniform registers
+  // and the 96-register cap no longer spills (SK N = 512 x 152: 16.7 -> 15.6 us per sweep).
+  const int grp = __shfl_sync(0xFFFFFFFFu, epi ? (warp - 2) >> 2 : 0, 0);
   const int row = quad * 32 + lane;             // replica row inside the panel
   const uint32_t full0 = smem_u32(&bars[0]);
   const uint32_t empty0 = smem_u32(&bars[kStages]);
@@ -240,6 +251,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
   const uint32_t tempty0 = smem_u32(&bars[2 * kStages + kBufs]);
   const uint32_t aready = smem_u32(&bars[2 * kStages + 2 * kBufs]);
   const uint32_t drain = aready + 8;
+  const uint32_t bar_tab0 = aready + 16;  // [2]
 
   if (warp == 1) {
     tmem_alloc(smem_u32(sTmem), kTmemCols);
@@ -256,6 +268,8 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
     }
     mbar_init(aready, 1);
     mbar_init(drain, 1);
+    mbar_init(bar_tab0, 1);
+    mbar_init(bar_tab0 + 8, 1);
     fence_mbar_init();
     *sAbort = 0;
   }
@@ -267,6 +281,8 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
 
   // Role counters, continued across units so every mbarrier phase is tracked exactly.
   uint32_t loads = 0, mmas = 0, cpass = 0, apass = 0;
+  uint32_t tabs_copied = 0;  // MMA warp: every table copy it has issued
+  uint32_t tabs = 0;  // tables copied ahead in earlier units (table k lies in half k & 1)
   bool first_unit = true;
   const uint32_t idesc = idesc_e4m3(128, kNT);
 
@@ -281,6 +297,10 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
     const int n = P.n, npad = P.npad, R = P.R;
     const int nchunks = npad / kNT, kblocks = npad / 128;
     const int t_begin = L.t_begin, t_end = L.t_begin + L.sweeps;
+    const int dk = DIAG ? P.dk : 0;
+    const int stride = dk > 0 ? 2 * dk : P.stride_words;  // table words per step
+    const uint32_t* thr = dk > 0 ? P.thr_diag : P.thr;
+    const bool tab_ahead = stride <= kTabHalf;
 
     if (warp == 0) {
       // ---- producer (converged warp, one elected lane): coupling K-blocks into the ring ---
@@ -325,6 +345,17 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
       const uint32_t idesc_u = P.e5m2 ? idesc_e5m2(128, kNT) : idesc;
       const uint64_t ring_desc = sw128_desc(smem_u32(sRing));
       bool ok = true;
+      auto copy_table = [&](int t) {  // table of step t into its half
+        const uint32_t k = tabs + static_cast<uint32_t>(t - t_begin), half = k & 1;
+        if (elect_one()) {
+          mbar_expect_tx(bar_tab0 + 8 * half, stride * 4);
+          bulk_g2s(smem_u32(sTab) + half * kTabHalf * 4, thr + static_cast<size_t>(t) * stride, stride * 4,
+                   bar_tab0 + 8 * half);
+        }
+        __syncwarp();
+        tabs_copied = k + 1;
+      };
+      if (tab_ahead && t_begin < t_end) copy_table(t_begin);
       for (int t = t_begin; t <= t_end && ok; ++t) {
         if (!__all_sync(0xFFFFFFFFu, wait_phase(aready, apass & 1, L.wait_ns))) {
           ok = false;
@@ -332,6 +363,8 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
         }
         ++apass;
         tc_fence_after();
+        // sweep t - 1 is decided: its table's half takes the next step's
+        if (tab_ahead && t + 1 < t_end) copy_table(t + 1);
         for (int c = 0; c < nchunks && ok; ++c) {
           const uint32_t b = cpass % kBufs, buse = cpass / kBufs;
           if (!__all_sync(0xFFFFFFFFu, buse == 0 || wait_phase(tempty0 + 8 * b, (buse - 1) & 1, L.wait_ns))) {
@@ -420,32 +453,40 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
 
       // Problem fields in registers: the loops below store to global memory, which would
       // otherwise make the compiler reload them from the descriptor.
-      const uint32_t q = P.q;
-      const int dk = DIAG ? P.dk : 0;
-      const int imax = P.imax, stride = dk > 0 ? 2 * dk : P.stride_words;  // words per step
-      const uint32_t* thr = dk > 0 ? P.thr_diag : P.thr;
+      const uint32_t q = __shfl_sync(0xFFFFFFFFu, P.q, 0);
+      const int imax = P.imax;
       const long long target = P.target;
       const bool tab_smem = stride <= kTabWords;
       const bool has_target = P.has_target != 0;
       const int dg = P.diag_img ? 256 : 0;  // diagonal-encoded image: D = I + 256 s
       const bool fast = !DIAG && P.h == nullptr && !P.diag_img && tab_smem;
       constexpr bool dfast = DIAG;  // diagonal-encoded table in shared memory (2 dk <= kTabWords)
-      // byte address of the entry of D: 2 (bits of D + 1.5*2^23) + tab_d (mod 2^32)
-      const uint32_t tab_d = smem_u32(sTab) + 4u * static_cast<uint32_t>(dk) - 2u * kMagicBits;
       const int e_off = dfast ? dk * n : 0;  // sum of |D| over the n spins = sum s I + n dk
-      const uint32_t tab_c = smem_u32(sTab) + 4u * static_cast<uint32_t>(imax) - 4u * kMagicBits;  // mod 2^32
       for (int t = t_begin; t <= t_end && !stop; ++t) {
         const bool last = t == t_end;
-        if (tab_smem && !last) {
-          const uint4* src = reinterpret_cast<const uint4*>(thr + static_cast<size_t>(t) * stride);
-          for (int k = etid; k < stride / 4; k += kEpiThreads)
-            reinterpret_cast<uint4*>(sTab)[k] = __ldg(src + k);
-        }
-        if (bar_sync_or(1, kEpiThreads, *sAbort != 0)) break;
-        const uint32_t* tab =
-            tab_smem ? sTab : thr + static_cast<size_t>(last ? t_begin : t) * stride;
-        int eacc = 0;
         bool waitfail = false;
+        uint32_t half = 0;
+        if (tab_ahead) {
+          const uint32_t k = tabs + static_cast<uint32_t>(t - t_begin);
+          half = k & 1;
+          if (!last && !wait_phase(bar_tab0 + 8 * half, (k >> 1) & 1, L.wait_ns)) waitfail = true;
+        } else {
+          if (tab_smem && !last) {
+            const uint4* src = reinterpret_cast<const uint4*>(thr + static_cast<size_t>(t) * stride);
+            for (int k = etid; k < stride / 4; k += kEpiThreads)
+              reinterpret_cast<uint4*>(sTab)[k] = __ldg(src + k);
+            fence_proxy_async_smem();  // a later unit's bulk copies may take the same words
+          }
+          if (bar_sync_or(1, kEpiThreads, *sAbort != 0)) break;
+        }
+        const uint32_t* tab =
+            tab_smem ? sTab + half * kTabHalf : thr + static_cast<size_t>(last ? t_begin : t) * stride;
+        const uint32_t tab_at = smem_u32(sTab) + half * kTabHalf * 4;
+        // byte address of the entry of D: 2 (bits of D + 1.5*2^23) + tab_d (mod 2^32)
+        const uint32_t tab_d = tab_at + 4u * static_cast<uint32_t>(dk) - 2u * kMagicBits;
+        const uint32_t tab_c = tab_at + 4u * static_cast<uint32_t>(imax) - 4u * kMagicBits;  // mod 2^32
+        int* red = sRed + (t & 1) * kGroups * 128;
+        int eacc = 0;
 #pragma unroll 1
         for (int c = 0; c < nchunks; ++c) {
           const uint32_t b = cpass % kBufs, buse = cpass / kBufs;
@@ -553,7 +594,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
           tmem_wait_st();
           tc_fence_before();
         }
-        sRed[grp * 128 + row] = eacc;
+        red[grp * 128 + row] = eacc;
         stop = bar_sync_or(1, kEpiThreads, waitfail || *sAbort != 0);
         if (stop) {
           if (etid == 0) {
@@ -565,7 +606,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
         if (!last && etid == 0) mbar_arrive(aready);
         int tot = 0;
 #pragma unroll
-        for (int g = 0; g < kGroups; ++g) tot += sRed[g * 128 + row];
+        for (int g = 0; g < kGroups; ++g) tot += red[g * 128 + row];
         const int E = -((tot - e_off) / 2);
         if (E < best_E) {
           // the best state lives in the output array: written when it improves
@@ -603,12 +644,15 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
       }
     }
     first_unit = false;
+    if (tab_ahead) tabs += L.sweeps;
   }
 
   // ---- teardown: no copy or MMA of this CTA may still be in flight ------------------------
   if (tid == 32) {
     mma_commit(drain);
     wait_phase(drain, 0, L.wait_ns);
+    for (uint32_t k = tabs_copied > 2 ? tabs_copied - 2 : 0; k < tabs_copied; ++k)
+      wait_phase(bar_tab0 + 8 * (k & 1), (k >> 1) & 1, L.wait_ns);
   } else if (tid == 0) {
     for (uint32_t k = loads > kStages ? loads - kStages : 0; k < loads; ++k)
       wait_phase(full0 + 8 * (k % kStages), (k / kStages) & 1, L.wait_ns);
@@ -621,7 +665,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
 }  // namespace
 
 int sweep_mid_smem_bytes() {
-  return 1024 + kStages * kStageBytes + kTabWords * 4 + kGroups * 128 * 4 + kMaxNpad * 4 +
+  return 1024 + kStages * kStageBytes + kTabWords * 4 + 2 * kGroups * 128 * 4 + kMaxNpad * 4 +
          kBarCount * 8 + 32;
 }
 
