@@ -37,6 +37,7 @@
 #include <climits>
 #include <type_traits>
 
+#include "int_rule.cuh"
 #include "kernels.h"
 #include "philox.cuh"
 #include "real_rule.cuh"
@@ -604,7 +605,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_big_kernel(const __grid_con
                 auto decide = [&](int e, uint32_t th) {
                   const uint32_t word = rw[8 * c + (e >> 1)];
                   const uint32_t d = (e & 1) ? (word >> 16) : (word & 0xFFFFu);
-                  neg = __funnelshift_l(d + th * 0xFFFFFFF0u, neg, 1);
+                  neg = __funnelshift_l(draw_below(d, th, e & 1), neg, 1);
                 };
                 if (tab_smem) {
                   const uint32_t tab_c = smem_u32(sTab) + 4u * static_cast<uint32_t>(P.imax) - 4u * kMagicBits;

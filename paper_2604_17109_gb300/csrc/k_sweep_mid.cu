@@ -25,6 +25,7 @@
 //            it improves) and first hit per replica.
 #include <climits>
 
+#include "int_rule.cuh"
 #include "kernels.h"
 #include "philox.cuh"
 #include "sm100_ptx.cuh"
@@ -82,99 +83,13 @@ __device__ __forceinline__ void put_spins32_tm(uint32_t tlane, int col, uint32_t
 constexpr float kMagic = 12582912.0f;      // 1.5 * 2^23: integer D in the low mantissa bits
 constexpr uint32_t kMagicBits = 0x4B400000u;
 
-// Bits of (a + 1.5 * 2^23) and (b + 1.5 * 2^23) for two exactly integral fields in one
-// packed FP32 add (round to nearest: identical to two scalar adds, exact for |D| < 2^22).
-__device__ __forceinline__ void magic_add2(uint32_t a, uint32_t b, uint32_t& va, uint32_t& vb) {
-  uint64_t pr, rr;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(pr) : "r"(a), "r"(b));
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(rr) : "l"(pr), "l"(0x4B4000004B400000ull));
-  asm("mov.b64 {%0, %1}, %2;" : "=r"(va), "=r"(vb) : "l"(rr));
-}
-
-// Sixteen spins of one replica, general-bias table without bias (h = 0, plain image):
-// vb = bits(D + 1.5 * 2^23) = 0x4B400000 + I, the 16-bit threshold of (s, I) at shared
-// address tab_c + 4 vb + 2 s (tab_c = table + 4 (imax - 0x4B400000), mod 2^32), and
-// key >= M  <=>  d >= 16 M for the 16-bit draw d (key = d >> 4); the sign bits of d - 16 M
-// (new spin -1) are shifted in by two chains.  sum_all / sum_up collect vb over all spins /
-// the +1 spins for the energy.  Returns the new spins as bits 0..15.
-template <bool DECIDE>
-__device__ __forceinline__ uint32_t bias_chunk16(const uint32_t (&v)[16], const uint32_t (&rw)[8],
-                                                 uint32_t cw16, uint32_t tab_c, uint32_t& sum_all,
-                                                 uint32_t& sum_up) {
-  uint32_t neg_hi = 0, neg_lo = 0, sa = 0, su = 0;
-  uint32_t vpair = 0;
-#pragma unroll
-  for (int e = 15; e >= 0; --e) {
-    uint32_t vb;
-    if (e & 1)
-      magic_add2(v[e - 1], v[e], vpair, vb);
-    else
-      vb = vpair;
-    const uint32_t s = (cw16 >> e) & 1u;
-    sa += vb;
-    su += s * vb;
-    if constexpr (DECIDE) {
-      uint32_t m;
-      asm volatile("ld.shared.u16 %0, [%1];" : "=r"(m) : "r"(tab_c + 4u * vb + 2u * s));
-      const uint32_t w = rw[e >> 1];
-      const uint32_t d = (e & 1) ? (w >> 16) : (w & 0xFFFFu);
-      const uint32_t diff = d + m * 0xFFFFFFF0u;  // d - 16 m
-      if (e >= 8)
-        neg_hi = __funnelshift_l(diff, neg_hi, 1);
-      else
-        neg_lo = __funnelshift_l(diff, neg_lo, 1);
-    }
-  }
-  sum_all += sa;
-  sum_up += su;
-  return ~((neg_hi << 8) | neg_lo) & 0xFFFFu;
-}
-
-// Sixteen spins of one replica, diagonal-encoded image (D = I + dk s, |I| < dk, h = 0): the
-// 16-bit threshold of (s, I) is the table entry of D at shared address 2 vb + tab_d
-// (vb = bits(D + 1.5 * 2^23), tab_d = table + 2 (2 dk) - 2 * 0x4B400000, mod 2^32), and
-// |D| = s I + dk sums to the energy.  Returns the new spins as bits 0..15.
-template <bool DECIDE>
-__device__ __forceinline__ uint32_t diag_chunk16(const uint32_t (&v)[16], const uint32_t (&rw)[8],
-                                                 uint32_t tab_d, float& esum) {
-  uint32_t neg_hi = 0, neg_lo = 0;
-  float e_a = 0.0f, e_b = 0.0f;
-  uint32_t vpair = 0;
-#pragma unroll
-  for (int e = 15; e >= 0; --e) {
-    const float fd = __uint_as_float(v[e]);
-    if constexpr (DECIDE) {
-      uint32_t vb;
-      if (e & 1)
-        magic_add2(v[e - 1], v[e], vpair, vb);
-      else
-        vb = vpair;
-      uint32_t m;
-      asm volatile("ld.shared.u16 %0, [%1];" : "=r"(m) : "r"(vb * 2u + tab_d));
-      const uint32_t w = rw[e >> 1];
-      const uint32_t d = (e & 1) ? (w >> 16) : (w & 0xFFFFu);
-      const uint32_t diff = d + m * 0xFFFFFFF0u;  // d - 16 m
-      if (e >= 8)
-        neg_hi = __funnelshift_l(diff, neg_hi, 1);
-      else
-        neg_lo = __funnelshift_l(diff, neg_lo, 1);
-    }
-    if (e & 1)
-      e_a += fabsf(fd);
-    else
-      e_b += fabsf(fd);
-  }
-  esum += e_a + e_b;
-  return ~((neg_hi << 8) | neg_lo) & 0xFFFFu;
-}
-
-// A thread's 32 columns of one chunk (two 16-column halves): the TMEM load of each half runs
-// while its two Philox blocks are drawn (DECIDE: every sweep but the final energy pass),
-// then diag_chunk16 / bias_chunk16.  Returns the new spins of the 32 columns as bits.
-template <bool DECIDE>
-__device__ __forceinline__ uint32_t diag_chunk32(uint32_t ta, uint32_t blk0, uint32_t rg, uint32_t t,
-                                                 uint32_t q, const uint32_t* rk, uint32_t tab_d,
-                                                 float& esum) {
+// A thread's 32 columns of one chunk (two 16-column halves): the TMEM load of each half runs while its
+// two Philox blocks are drawn (DECIDE: every sweep but the final energy pass), then the rule.  Returns
+// the new spins of the 32 columns as bits.
+template <bool DIAG, bool DECIDE>
+__device__ __forceinline__ uint32_t chunk32(uint32_t ta, uint32_t blk0, uint32_t rg, uint32_t t, uint32_t q,
+                                            const uint32_t* rk, uint32_t cw32, const int* h, uint32_t base,
+                                            float& esum) {
   uint32_t word = 0;
 #pragma unroll
   for (int h2 = 0; h2 < 2; ++h2) {
@@ -187,44 +102,59 @@ __device__ __forceinline__ uint32_t diag_chunk32(uint32_t ta, uint32_t blk0, uin
     }
     tmem_wait_ld(v);
     const uint32_t rw8[8] = {o0.x0, o0.x1, o0.x2, o0.x3, o1.x0, o1.x1, o1.x2, o1.x3};
-    word |= diag_chunk16<DECIDE>(v, rw8, tab_d, esum) << (16 * h2);
+    if constexpr (DIAG)
+      word |= diag_rule<16>(v, rw8, base, esum, DECIDE) << (16 * h2);
+    else
+      word |= bias_rule<16>(v, rw8, (cw32 >> (16 * h2)) & 0xFFFFu, reinterpret_cast<const float*>(h) + 16 * h2,
+                            base, esum, DECIDE)
+              << (16 * h2);
   }
   return word;
 }
 
-// As diag_chunk32 for the general table without bias (h = 0, plain image); cw32 holds the
-// 32 current spins, eacc collects sum_i s_i I_i.
-template <bool DECIDE>
-__device__ __forceinline__ uint32_t bias_chunk32(uint32_t ta, uint32_t blk0, uint32_t rg, uint32_t t,
-                                                 uint32_t q, const uint32_t* rk, uint32_t cw32,
-                                                 uint32_t tab_c, int& eacc) {
+// The same columns with the table in global memory (imax >= 2048), or of a diagonal-encoded image
+// without its table.  Out of line: inlined, its sixteen table reads in flight spill the loop around it.  Returns the spins and the energy sum.
+__device__ __forceinline__ uint32_t table_chunk32(uint32_t ta, int col0, int n, const int* sH, int dg, uint32_t cw32,
+                                               const uint16_t* tab16, bool last, uint32_t rg, uint32_t t,
+                                               uint32_t q, const uint32_t* rk, int& eacc) {
   uint32_t word = 0;
-#pragma unroll
+#pragma unroll 1
   for (int h2 = 0; h2 < 2; ++h2) {
     uint32_t v[16];
     tmem_ld16(ta + 16 * h2, v);
-    PhiloxOut o0{}, o1{};
-    if constexpr (DECIDE) {
-      o0 = philox4x32_10_rk(blk0 + 2 * h2, rg, t, q, rk);
-      o1 = philox4x32_10_rk(blk0 + 2 * h2 + 1, rg, t, q, rk);
-    }
+    const uint32_t blk = static_cast<uint32_t>(col0 >> 3) + 2 * h2;
+    const PhiloxOut o0 = philox4x32_10_rk(blk, rg, t, q, rk), o1 = philox4x32_10_rk(blk + 1, rg, t, q, rk);
     tmem_wait_ld(v);
     const uint32_t rw8[8] = {o0.x0, o0.x1, o0.x2, o0.x3, o1.x0, o1.x1, o1.x2, o1.x3};
-    const uint32_t cw16 = (cw32 >> (16 * h2)) & 0xFFFFu;
-    uint32_t sa = 0, su = 0;
-    const uint32_t nb = bias_chunk16<DECIDE>(v, rw8, cw16, tab_c, sa, su);
-    eacc += static_cast<int>(2u * (su - static_cast<uint32_t>(__popc(cw16)) * kMagicBits) -
-                             (sa - 16u * kMagicBits));
-    word |= nb << (16 * h2);
+    const uint32_t cw16 = cw32 >> (16 * h2);
+    uint32_t th[16], neg = 0;
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+      const int col = col0 + 16 * h2 + e;
+      const int s = static_cast<int>((cw16 >> e) & 1u);
+      const int hv = sH[col];
+      const int dgc = col < n ? (s ? dg : -dg) : 0;  // image diagonal inside n only
+      // exact float -> int of the integer-valued field (|D| < 2^22)
+      const int I = static_cast<int>(__float_as_uint(__fadd_rn(__uint_as_float(v[e]), kMagic)) - kMagicBits) +
+                    hv - dgc;
+      const int term = I + hv;
+      eacc += s ? term : -term;
+      th[e] = last ? 0 : __ldg(tab16 + 2 * I + s);
+    }
+#pragma unroll
+    for (int e = 15; e >= 0; --e) neg = __funnelshift_l(draw_below(draw_of(rw8, e), th[e], true), neg, 1);
+    word |= (~neg & 0xFFFFu) << (16 * h2);
   }
   return word;
 }
 
-// DIAG = true: every unit has a diagonal-encoded image (P.dk > 0) and decides from its
-// 16-bit table; DIAG = false: no unit has one (bias fast path or general path).  Two
-// variants keep the register allocation of each to the paths it runs.
-template <bool DIAG>
+// One variant per MidMode keeps the register allocation of each to the path that it runs.  One kernel
+// for both general tables took 30.2 us per sweep at N = 400 with a bias (80 instances x 256 replicas)
+// and 23.7 at N = 700 with couplings of +-9 and a bias (60 x 256); these take 17.1 and 20.1, and a bias
+// unit beside one with a larger table, on the variant for global memory, 27.3.
+template <int MODE>
 __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_constant__ Launch L) {
+  constexpr bool DIAG = MODE == kMidDiag;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -300,7 +230,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
     const int dk = DIAG ? P.dk : 0;
     const int stride = dk > 0 ? 2 * dk : P.stride_words;  // table words per step
     const uint32_t* thr = dk > 0 ? P.thr_diag : P.thr;
-    const bool tab_ahead = stride <= kTabHalf;
+    const bool tab_ahead = MODE != kMidTable && stride <= kTabHalf;
 
     if (warp == 0) {
       // ---- producer (converged warp, one elected lane): coupling K-blocks into the ring ---
@@ -438,7 +368,10 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
         best_t = P.best_t[rg];
         first_hit = P.first_hit[rg];
       }
-      for (int k = etid; k < npad; k += kEpiThreads) sH[k] = (P.h != nullptr && k < n) ? P.h[k] : 0;
+      for (int k = etid; !DIAG && k < npad; k += kEpiThreads) {
+        const int hv = (P.h != nullptr && k < n) ? P.h[k] : 0;
+        sH[k] = MODE == kMidBias ? __float_as_int(static_cast<float>(hv)) : hv;
+      }
 #pragma unroll
       for (int c = 0; c < kMaxChunks; ++c)
 #pragma unroll
@@ -456,12 +389,9 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
       const uint32_t q = __shfl_sync(0xFFFFFFFFu, P.q, 0);
       const int imax = P.imax;
       const long long target = P.target;
-      const bool tab_smem = stride <= kTabWords;
       const bool has_target = P.has_target != 0;
       const int dg = P.diag_img ? 256 : 0;  // diagonal-encoded image: D = I + 256 s
-      const bool fast = !DIAG && P.h == nullptr && !P.diag_img && tab_smem;
-      constexpr bool dfast = DIAG;  // diagonal-encoded table in shared memory (2 dk <= kTabWords)
-      const int e_off = dfast ? dk * n : 0;  // sum of |D| over the n spins = sum s I + n dk
+      const int e_off = DIAG ? dk * n : 0;  // sum of |D| over the n spins = sum s I + n dk
       for (int t = t_begin; t <= t_end && !stop; ++t) {
         const bool last = t == t_end;
         bool waitfail = false;
@@ -471,7 +401,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
           half = k & 1;
           if (!last && !wait_phase(bar_tab0 + 8 * half, (k >> 1) & 1, L.wait_ns)) waitfail = true;
         } else {
-          if (tab_smem && !last) {
+          if (MODE != kMidTable && !last) {
             const uint4* src = reinterpret_cast<const uint4*>(thr + static_cast<size_t>(t) * stride);
             for (int k = etid; k < stride / 4; k += kEpiThreads)
               reinterpret_cast<uint4*>(sTab)[k] = __ldg(src + k);
@@ -479,12 +409,10 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
           }
           if (bar_sync_or(1, kEpiThreads, *sAbort != 0)) break;
         }
-        const uint32_t* tab =
-            tab_smem ? sTab + half * kTabHalf : thr + static_cast<size_t>(last ? t_begin : t) * stride;
-        const uint32_t tab_at = smem_u32(sTab) + half * kTabHalf * 4;
-        // byte address of the entry of D: 2 (bits of D + 1.5*2^23) + tab_d (mod 2^32)
-        const uint32_t tab_d = tab_at + 4u * static_cast<uint32_t>(dk) - 2u * kMagicBits;
-        const uint32_t tab_c = tab_at + 4u * static_cast<uint32_t>(imax) - 4u * kMagicBits;  // mod 2^32
+        const uint16_t* tab16 =  // in global memory, entry of s = -1 and I = 0
+            reinterpret_cast<const uint16_t*>(thr + static_cast<size_t>(last ? t_begin : t) * stride + imax);
+        // byte address of the entry of D = 0, or of the one of s = -1 and I = 0
+        const uint32_t base = smem_u32(sTab) + half * kTabHalf * 4 + 4u * static_cast<uint32_t>(DIAG ? dk : imax);
         int* red = sRed + (t & 1) * kGroups * 128;
         int eacc = 0;
 #pragma unroll 1
@@ -495,87 +423,25 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
           tc_fence_after();
           const uint32_t ta = tmem + (static_cast<uint32_t>(quad * 32) << 16) + b * kNT + grp * kCols;
           const uint32_t blk0 = static_cast<uint32_t>((c * kNT + grp * kCols) >> 3);
-          if (dfast) {
-            // Diagonal-encoded fields, 16 columns at a time (diag_chunk16).
-            static_assert(kCols == 32 && kWordsPT == 1, "one 32-bit spin word per thread and chunk");
-            // Columns at or past n (the padding of the last chunk) have zero fields and stay
-            // -1: a thread whose 32 columns all lie there skips them (nxt stays 0).
-            if (warp_active && c * kNT + grp * kCols < n) {
+          static_assert(kCols == 32 && kWordsPT == 1, "one 32-bit spin word per thread and chunk");
+          uint32_t word = 0;  // new spins; columns at or past n stay -1 (bit 0)
+          const int col0 = c * kNT + grp * kCols;
+          // A thread whose 32 columns all lie at or past n skips them: their fields are zero, and they
+          // stay -1.
+          if (warp_active && col0 < n) {
+            if constexpr (MODE == kMidTable) {
+              word = table_chunk32(ta, col0, n, sH, dg, cur[c][0], tab16, last, static_cast<uint32_t>(rg),
+                                   static_cast<uint32_t>(t), q, L.round_keys, eacc);
+            } else {
               float esum = 0.0f;
-              const uint32_t word =
-                  last ? diag_chunk32<false>(ta, blk0, static_cast<uint32_t>(rg), static_cast<uint32_t>(t), q,
-                                             L.round_keys, tab_d, esum)
-                       : diag_chunk32<true>(ta, blk0, static_cast<uint32_t>(rg), static_cast<uint32_t>(t), q,
-                                            L.round_keys, tab_d, esum);
-              nxt[c][0] = word & valid_mask(c, 0);
+              word = last ? chunk32<DIAG, false>(ta, blk0, static_cast<uint32_t>(rg), static_cast<uint32_t>(t), q,
+                                                 L.round_keys, cur[c][0], sH + col0, base, esum)
+                          : chunk32<DIAG, true>(ta, blk0, static_cast<uint32_t>(rg), static_cast<uint32_t>(t), q,
+                                                L.round_keys, cur[c][0], sH + col0, base, esum);
               eacc += static_cast<int>(esum);
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(tempty0 + 8 * b);
-            continue;
           }
-          if (fast) {
-            // 16 columns at a time: the TMEM load runs while their two Philox blocks are
-            // drawn, then the decisions (bias_chunk16); the buffer is released at the end.
-            if (warp_active && c * kNT + grp * kCols < n) {
-              const uint32_t word =
-                  last ? bias_chunk32<false>(ta, blk0, static_cast<uint32_t>(rg), static_cast<uint32_t>(t), q,
-                                             L.round_keys, cur[c][0], tab_c, eacc)
-                       : bias_chunk32<true>(ta, blk0, static_cast<uint32_t>(rg), static_cast<uint32_t>(t), q,
-                                            L.round_keys, cur[c][0], tab_c, eacc);
-              nxt[c][0] = word & valid_mask(c, 0);
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(tempty0 + 8 * b);
-            continue;
-          }
-          // General path (bias, diagonal-encoded image or a table in global memory), 16
-          // columns at a time like the fast path.
-          if (warp_active) {
-#pragma unroll
-            for (int h2 = 0; h2 < kCols / 16; ++h2) {
-              uint32_t v[16];
-              tmem_ld16(ta + 16 * h2, v);
-              PhiloxOut o0{}, o1{};
-              if (!last) {
-                o0 = philox4x32_10_rk(blk0 + 2 * h2, static_cast<uint32_t>(rg),
-                                      static_cast<uint32_t>(t), q, L.round_keys);
-                o1 = philox4x32_10_rk(blk0 + 2 * h2 + 1, static_cast<uint32_t>(rg),
-                                      static_cast<uint32_t>(t), q, L.round_keys);
-              }
-              tmem_wait_ld(v);
-              const uint32_t rw8[8] = {o0.x0, o0.x1, o0.x2, o0.x3, o1.x0, o1.x1, o1.x2, o1.x3};
-              const int w = h2 >> 1;
-              const uint32_t cw16 = (cur[c][w] >> (16 * (h2 & 1))) & 0xFFFFu;
-              uint32_t nb = 0;
-#pragma unroll
-              for (int e = 0; e < 16; ++e) {
-                const int col = c * kNT + grp * kCols + 16 * h2 + e;
-                const uint32_t s = (cw16 >> e) & 1u;
-                const int hv = sH[col];
-                const int dgc = col < n ? (s ? dg : -dg) : 0;  // image diagonal inside n only
-                // exact float -> int of the integer-valued field (|D| < 2^22)
-                const int D = static_cast<int>(__float_as_uint(__fadd_rn(__uint_as_float(v[e]), kMagic)) -
-                                               kMagicBits);
-                const int I = D + hv - dgc;
-                const int term = I + hv;
-                eacc += s ? term : -term;
-                if (!last) {
-                  const uint32_t wd = tab[I + imax];
-                  const uint32_t th = s ? (wd >> 16) : (wd & 0xFFFFu);
-                  const uint32_t word = rw8[e >> 1];
-                  const uint32_t key = (e & 1) ? (word >> 20) : ((word >> 4) & 0xFFFu);
-                  nb |= (key >= th ? 1u : 0u) << e;
-                }
-              }
-              if (h2 & 1)
-                nxt[c][w] = (nxt[c][w] | (nb << 16)) & valid_mask(c, w);
-              else
-                nxt[c][w] = nb;
-            }
-          }
+          nxt[c][0] = word & valid_mask(c, 0);
           // TMEM buffer b drained by this warp: let the MMA issuer reuse it.
           tc_fence_before();
           __syncwarp();
@@ -673,11 +539,11 @@ int sweep_mid_max_npad() { return kMaxNpad; }
 
 int sweep_mid_max_blocks() {
   const int smem = sweep_mid_smem_bytes();
-  if (cudaFuncSetAttribute(sweep_mid_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
+  if (cudaFuncSetAttribute(sweep_mid_kernel<kMidTable>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
       cudaSuccess)
     return 0;
   int per_sm = 0, dev = 0, sms = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sweep_mid_kernel<false>, kThreads, smem) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sweep_mid_kernel<kMidTable>, kThreads, smem) !=
       cudaSuccess)
     return 0;
   cudaGetDevice(&dev);
@@ -685,17 +551,18 @@ int sweep_mid_max_blocks() {
   return per_sm * sms;
 }
 
-cudaError_t launch_sweep_mid(const Launch& L, int blocks, cudaStream_t st, bool diag) {
+int sweep_mid_table_words() { return kTabWords; }
+
+cudaError_t launch_sweep_mid(const Launch& L, int blocks, cudaStream_t st, MidMode mode) {
+  const auto kernel = mode == kMidDiag   ? sweep_mid_kernel<kMidDiag>
+                      : mode == kMidBias ? sweep_mid_kernel<kMidBias>
+                                         : sweep_mid_kernel<kMidTable>;
   const int smem = sweep_mid_smem_bytes();
-  cudaError_t e = cudaFuncSetAttribute(diag ? sweep_mid_kernel<true> : sweep_mid_kernel<false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(L.next, 0, sizeof(unsigned int), st);
   if (e != cudaSuccess) return e;
-  if (diag)
-    sweep_mid_kernel<true><<<blocks, kThreads, smem, st>>>(L);
-  else
-    sweep_mid_kernel<false><<<blocks, kThreads, smem, st>>>(L);
+  kernel<<<blocks, kThreads, smem, st>>>(L);
   return cudaGetLastError();
 }
 

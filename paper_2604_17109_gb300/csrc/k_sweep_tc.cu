@@ -16,6 +16,7 @@
 // replica is a thread-local sum plus the partial sums of the other column groups' threads.
 #include <climits>
 
+#include "int_rule.cuh"
 #include "kernels.h"
 #include "philox.cuh"
 #include "sm100_ptx.cuh"
@@ -26,12 +27,6 @@ namespace {
 constexpr int kGroups = 2;               // column groups of a replica row (2 or 3)
 constexpr int kThreads = 128 * kGroups;  // 4 TMEM lane quadrants x kGroups column groups
 constexpr int kTileM = 128;              // replicas per CTA (MMA M)
-
-// The integer value I of an exactly integral float f (|f| < 2^22) appears in the low
-// mantissa bits of f + 1.5 * 2^23.
-constexpr float kMagic = 12582912.0f;
-constexpr uint32_t kMagicBits = 0x4B400000u;
-constexpr uint64_t kMagicPair = 0x4B4000004B400000ull;  // two FP32 1.5 * 2^23
 
 // Two decision modes.
 //  kModeDiag: h = 0 and |I| <= 255.  The couplings are staged with 256 on the diagonal, so
@@ -63,7 +58,7 @@ static_assert(kGroups == 2 || kGroups == 3, "column split checked for 2 and 3 gr
 template <int W>
 __device__ __forceinline__ uint32_t diag_chunk(uint32_t taddr, uint32_t c, uint32_t rg,
                                                uint32_t t, uint32_t q, const uint32_t* rk,
-                                               uint32_t diag_bias, float& eacc) {
+                                               uint32_t diag_base, float& eacc) {
   uint32_t v[W];
   if constexpr (W == 16)
     tmem_ld16(taddr, v);
@@ -84,41 +79,7 @@ __device__ __forceinline__ uint32_t diag_chunk(uint32_t taddr, uint32_t c, uint3
     rw[7] = o1.x3;
   }
   tmem_wait_ld(v);
-  // Sign bits of (draw - 16 M) are shifted in from the top: after the last step bit e is set
-  // iff key(e) < M, i.e. the new spin is -1.  Two shift chains and two energy sums keep the
-  // dependent sequences short.
-  uint32_t neg_hi = 0, neg_lo = 0;
-  float e_a = 0.0f, e_b = 0.0f;
-  // bits of D + 1.5 * 2^23 for two spins per instruction (packed FP32 add, round to nearest:
-  // exact for these integers, identical to two scalar adds)
-  uint32_t ibv[W];
-#pragma unroll
-  for (int e = 0; e < W; e += 2) {
-    uint64_t pr, rr;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(pr) : "r"(v[e]), "r"(v[e + 1]));
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(rr) : "l"(pr), "l"(kMagicPair));
-    asm("mov.b64 {%0, %1}, %2;" : "=r"(ibv[e]), "=r"(ibv[e + 1]) : "l"(rr));
-  }
-#pragma unroll
-  for (int e = W - 1; e >= 0; --e) {
-    const float f = __uint_as_float(v[e]);
-    const uint32_t ib = ibv[e];
-    uint32_t m;
-    asm volatile("ld.shared.u16 %0, [%1];" : "=r"(m) : "r"(ib * 2u + diag_bias));
-    const uint32_t w = rw[e >> 1];
-    const uint32_t d = (e & 1) ? (w >> 16) : (w & 0xFFFFu);
-    const uint32_t diff = d + m * 0xFFFFFFF0u;  // d - 16 m
-    if (e >= W / 2)
-      neg_hi = __funnelshift_l(diff, neg_hi, 1);
-    else
-      neg_lo = __funnelshift_l(diff, neg_lo, 1);
-    if (e & 1)
-      e_a += fabsf(f);
-    else
-      e_b += fabsf(f);
-  }
-  eacc += e_a + e_b;
-  return ~((neg_hi << (W / 2)) | neg_lo) & ((1u << W) - 1u);
+  return diag_rule<W>(v, rw, diag_base, eacc);
 }
 
 // QUEUE = false: CTA b runs work item b, all sweeps.  QUEUE = true: persistent CTAs take
@@ -137,7 +98,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_tc_kernel(const Launch L) {
   uint8_t* sA = sJ + NPAD * NPAD;
   uint32_t* sT = reinterpret_cast<uint32_t*>(sA + kTileM * NPAD);
   float* sPart = reinterpret_cast<float*>(sT + 2 * SW);
-  int* sH = reinterpret_cast<int*>(sPart + 2 * kGroups * kTileM);
+  float* sH = sPart + 2 * kGroups * kTileM;
   uint64_t* bars = reinterpret_cast<uint64_t*>(sH + (MODE == kModeBias ? NPAD : 0));
   uint32_t* sTmem = reinterpret_cast<uint32_t*>(bars + 2);
   int* sAbort = reinterpret_cast<int*>(sTmem + 1);
@@ -231,7 +192,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_tc_kernel(const Launch L) {
     for (int k = tid; k < kTileM * NPAD / 16; k += kThreads)
       reinterpret_cast<uint4*>(sA)[k] = make_uint4(0, 0, 0, 0);
     if (MODE == kModeBias)
-      for (int k = tid; k < NPAD; k += kThreads) sH[k] = (P.h != nullptr && k < n) ? P.h[k] : 0;
+      for (int k = tid; k < NPAD; k += kThreads) sH[k] = (P.h != nullptr && k < n) ? static_cast<float>(P.h[k]) : 0.0f;
     if (t_end > t_begin) {
       const uint4* src = reinterpret_cast<const uint4*>(thr + static_cast<size_t>(t_begin) * stride);
       uint4* dst = reinterpret_cast<uint4*>(sT + (t_begin & 1) * SW);
@@ -323,8 +284,6 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_tc_kernel(const Launch L) {
     jphase ^= 1u;
     __syncthreads();
     aborted = *sAbort != 0;
-    // kModeBias: word index of field I is (bits of I + 1.5*2^23) - (0x4B400000 - imax).
-    const uint32_t ioff = kMagicBits - static_cast<uint32_t>(imax);
 
     // ---- sweep loop ----------------------------------------------------------------------
     for (int t = t_begin; t < t_end && !aborted; ++t) {
@@ -345,8 +304,8 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_tc_kernel(const Launch L) {
         if (do_pre && k < stride / 4) pre[j] = __ldg(pre_src + k);
       }
       const uint32_t* tab = sT + (t & 1) * SW;
-      // kModeDiag: byte address of entry D is 2 * (bits of D + 1.5*2^23) + this bias (mod 2^32).
-      const uint32_t diag_bias = smem_u32(tab) + 2u * (kDiagEntries / 2) - 2u * kMagicBits;
+      const uint32_t diag_base = smem_u32(tab) + 2u * (kDiagEntries / 2);           // entry of D = 0
+      const uint32_t bias_base = smem_u32(tab) + 4u * static_cast<uint32_t>(imax);  // entry of s = -1, I = 0
       uint32_t nxt[kWordsPerThread];
 #pragma unroll
       for (int w = 0; w < kWordsPerThread; ++w) nxt[w] = 0;
@@ -360,12 +319,12 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_tc_kernel(const Launch L) {
             uint32_t nb;
             if (MODE == kModeDiag) {
               if (valid > 8) {
-                nb = diag_chunk<16>(tmem_warp + c * 16, c, rg, t, q, L.round_keys, diag_bias, eacc);
+                nb = diag_chunk<16>(tmem_warp + c * 16, c, rg, t, q, L.round_keys, diag_base, eacc);
                 if (valid < 16) nb &= (1u << valid) - 1u;
                 *reinterpret_cast<uint4*>(sA + sw128_offset(row, c * 16, kTileM)) =
                     fp8x16_from_bits(nb);
               } else {  // last chunk with at most 8 spins: half the work
-                nb = diag_chunk<8>(tmem_warp + c * 16, c, rg, t, q, L.round_keys, diag_bias, eacc);
+                nb = diag_chunk<8>(tmem_warp + c * 16, c, rg, t, q, L.round_keys, diag_base, eacc);
                 if (valid < 8) nb &= (1u << valid) - 1u;
                 *reinterpret_cast<uint2*>(sA + sw128_offset(row, c * 16, kTileM)) =
                     make_uint2(fp8x4_from_bits(nb & 0xFu), fp8x4_from_bits((nb >> 4) & 0xFu));
@@ -380,20 +339,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_tc_kernel(const Launch L) {
               tmem_wait_ld(v);
               const uint32_t rw[8] = {o0.x0, o0.x1, o0.x2, o0.x3, o1.x0, o1.x1, o1.x2, o1.x3};
               const uint32_t ob = (cur[k >> 1] >> ((k & 1) * 16)) & 0xFFFFu;
-              nb = 0;
-#pragma unroll
-              for (int e = 0; e < 16; ++e) {
-                const int hv = sH[c * 16 + e];
-                const uint32_t ib = __float_as_uint(__fadd_rn(__uint_as_float(v[e]), kMagic)) + hv;
-                const uint32_t w = tab[ib - ioff];
-                const uint32_t s = (ob >> e) & 1u;
-                const uint32_t th = s ? (w >> 16) : (w & 0xFFFFu);
-                const uint32_t word = rw[e >> 1];
-                const uint32_t key = (e & 1) ? (word >> 20) : ((word >> 4) & 0xFFFu);
-                nb |= (key >= th ? 1u : 0u) << e;
-                const int term = static_cast<int>(ib - kMagicBits) + hv;
-                eacc += static_cast<float>(s ? term : -term);
-              }
+              nb = bias_rule<16>(v, rw, ob, sH + c * 16, bias_base, eacc);
               if (valid < 16) nb &= (1u << valid) - 1u;
               *reinterpret_cast<uint4*>(sA + sw128_offset(row, c * 16, kTileM)) =
                   fp8x16_from_bits(nb);
@@ -455,16 +401,10 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_tc_kernel(const Launch L) {
           tmem_ld16(tmem_warp + c * 16, v);
           tmem_wait_ld(v);
           const uint32_t ob = (cur[k >> 1] >> ((k & 1) * 16)) & 0xFFFFu;
-#pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            if (MODE == kModeDiag) {
-              eacc += fabsf(__uint_as_float(v[e]));
-            } else {
-              const int term = static_cast<int>(__float_as_uint(__fadd_rn(__uint_as_float(v[e]), kMagic)) -
-                                                kMagicBits) + 2 * sH[c * 16 + e];
-              eacc += static_cast<float>(((ob >> e) & 1u) ? term : -term);
-            }
-          }
+          if (MODE == kModeDiag)
+            diag_rule<16>(v, nullptr, 0, eacc, false);
+          else
+            bias_rule<16>(v, nullptr, ob, sH + c * 16, 0, eacc, false);
         }
       }
     }

@@ -104,8 +104,13 @@ int sweep_big_max_blocks(int nt, int op, int npad, int stride_words);
 
 // Persistent mid-N kernel (integer couplings, npad <= 1024): `blocks` CTAs take the units
 // of L.work from the counter L.next (zeroed by the launch).
-// diag: every unit has P.dk > 0 (diagonal-encoded variant), else none has.
-cudaError_t launch_sweep_mid(const Launch& L, int blocks, cudaStream_t st, bool diag);
+// Every unit of a launch decides the same way: from a diagonal-encoded image and its 16-bit table
+// (P.dk > 0), from a general table that fits shared memory (a plain image, a step's table of at most
+// sweep_mid_table_words() words), or from a general table in global memory, which serves any unit with
+// P.dk = 0.
+enum MidMode { kMidTable = 0, kMidDiag = 1, kMidBias = 2 };
+cudaError_t launch_sweep_mid(const Launch& L, int blocks, cudaStream_t st, MidMode mode);
+int sweep_mid_table_words();
 int sweep_mid_max_blocks();
 int sweep_mid_max_npad();
 

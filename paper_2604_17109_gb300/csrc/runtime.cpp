@@ -1627,6 +1627,7 @@ struct BatchPlan {
   int rows[kGroups];  // replicas per work item
   int nmax[kGroups] = {};       // largest n of a group
   bool lat[kGroups] = {};       // integer fused groups: latency kernel
+  bool mid_bias = true;         // every unit of kMidGroup has its table in shared memory
   int maxR = 0, max_words = 0, stride_max = 4;
   size_t work_off[kGroups] = {};
   size_t ready_off[kGroups] = {};  // fused groups: chunked-queue counter and ready flags
@@ -1799,6 +1800,8 @@ int build_plan(pim_instance* const* insts, int count, const int* replicas, const
       continue;
     }
     const int g = group_of(k);
+    if (g == kMidGroup && (B.probs[k].diag_img || B.probs[k].stride_words > sweep_mid_table_words()))
+      B.mid_bias = false;
     for (int rb = 0; rb < replicas[k]; rb += B.rows[g]) B.work[g].push_back({k, rb});
   }
   // persistent launch: largest units first so the last wave is short
@@ -1909,7 +1912,8 @@ int enqueue_plan(const BatchPlan& B, char* d_buf, char* big_scratch, pim_instanc
       if (g == kMidGroup || g == kMidDiagGroup) {
         const int blocks = std::min(L.nwork, sweep_mid_max_blocks());
         if (blocks < 1) return fail(PIM_ERR_CUDA, "anneal: mid-N kernel cannot be resident");
-        CK(launch_sweep_mid(L, blocks, st, g == kMidDiagGroup), "persistent mid-N sweep kernel");
+        const MidMode mode = g == kMidDiagGroup ? kMidDiag : B.mid_bias ? kMidBias : kMidTable;
+        CK(launch_sweep_mid(L, blocks, st, mode), "persistent mid-N sweep kernel");
       } else if (g >= kRealGroup) {
         CK(launch_sweep_float(L, kRealCap[g - kRealGroup], g == kFixedGroup, L.nwork, st),
            "real-valued sweep kernel");

@@ -29,12 +29,14 @@ CASES = [(300, 0), (300, 1023), (300, 1024), (300, 2047), (300, 2048), (512, 0),
          (1000, 0), (1024, 0)]
 
 
+@pytest.mark.parametrize("shared", [False, True])
 @pytest.mark.parametrize("T", [1, 2, 7])
-def test_tables_in_one_batch(T):
-    """Every kind of unit follows another on the same SM, and each equals the oracle's run."""
+def test_tables_in_one_batch(T, shared):
+    """Every kind of unit follows another on the same SM, and each equals the oracle's run; with and
+    without units whose table is too large for shared memory."""
     P = pim()
     beta = linear_beta(T) if T > 1 else np.array([0.7])
-    insts = [_instance(n, imax) for n, imax in CASES]
+    insts = [_instance(n, imax) for n, imax in CASES if not shared or imax < 2048]
     R = (3, 130)[T % 2]
     hd = []
     try:
