@@ -17,9 +17,10 @@
 //            while the epilogue decides chunk c;
 //   decision 16 epilogue warps (4 TMEM lane quadrants x 4 groups of 32 columns): each
 //            thread owns one replica and 32 spins of every chunk, keeps their old / new
-//            bits in registers, draws the Philox blocks and looks the threshold up in the
-//            step's table at I = D + h; after the last chunk it writes the new spins into
-//            the tensor-memory A image (all MMAs of the sweep have completed by then);
+//            bits, draws the Philox blocks and looks the threshold up in the step's table at
+//            I = D + h (int_rule.cuh); the new spins go into a second tensor-memory image
+//            chunk by chunk (npad <= 512) or into the one image after the last chunk (all
+//            MMAs of the sweep have completed by then);
 //   energy   E(s(t)) = -1/2 sum_i s_i (I_i + h_i), exact in int32, reduced over the four
 //            column groups in shared memory; best state (written to the output array when
 //            it improves) and first hit per replica.
@@ -55,12 +56,20 @@ constexpr int kEpiThreads = kEpiWarps * 32;
 constexpr int kThreads = kEpiThreads + 64;  // + producer warp + MMA warp
 constexpr int kTmemA = kBufs * kNT;         // first TMEM column of the spin image (npad / 4 columns)
 constexpr int kTmemCols = kTmemA + kMaxNpad / 4;
+// Up to this npad two spin images fit: the new spins of a chunk go into the other image as soon as
+// they are decided, and the MMAs of the next sweep's first chunk run on all K-blocks but the last
+// while the last chunk is decided.  With one image the warps wrote a whole panel's spins after the last
+// chunk and then waited for a chunk's MMAs: SK N = 512 x 152 14.4 -> 13.4 us per sweep, N = 400 with a
+// bias, 80 x 256, 17.1 -> 16.3.
+constexpr int kTwoImages = kMaxNpad / 2;
+constexpr int kImageCols = kTwoImages / 4;
 constexpr int kBlockBytes = kNT * 128;      // one K-block of 128 coupling rows
 // K-blocks per ring stage: a bulk copy costs about the same producer and copy-engine time
 // whatever its size, so fewer, larger copies stream the couplings faster (measured: 4 x 3
 // stages beat 2 x 6, 3 x 4 and 6 x 2 on the uneven batch).
 constexpr int kKPS = 4;
 constexpr int kStageBytes = kKPS * kBlockBytes;
+static_assert(kTwoImages <= kKPS * 128, "with two images a chunk's K-blocks lie in one ring stage");
 constexpr int kBarCount = 2 * kStages + 2 * kBufs + 4;
 
 // Bounded wait with the common case (phase already complete) inline; the out-of-line wait
@@ -231,6 +240,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
     const int stride = dk > 0 ? 2 * dk : P.stride_words;  // table words per step
     const uint32_t* thr = dk > 0 ? P.thr_diag : P.thr;
     const bool tab_ahead = MODE != kMidTable && stride <= kTabHalf;
+    const bool two_images = npad <= kTwoImages;
 
     if (warp == 0) {
       // ---- producer (converged warp, one elected lane): coupling K-blocks into the ring ---
@@ -287,15 +297,49 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
       };
       if (tab_ahead && t_begin < t_end) copy_table(t_begin);
       for (int t = t_begin; t <= t_end && ok; ++t) {
-        if (!__all_sync(0xFFFFFFFFu, wait_phase(aready, apass & 1, L.wait_ns))) {
-          ok = false;
-          break;
+        const uint32_t a_img = tmem + kTmemA + (two_images ? (t & 1) * kImageCols : 0);
+        int c = 0;
+        if (two_images && t > t_begin) {
+          // First chunk.  Its accumulator is free once all chunks of sweep t - 1 but the last are
+          // decided, and so are all K-blocks of the new image but the last.
+          const uint32_t b = cpass % kBufs, buse = cpass / kBufs, p = cpass - 1;
+          const uint32_t s = mmas % kStages, use = mmas / kStages;
+          ok = __all_sync(0xFFFFFFFFu, (buse == 0 || wait_phase(tempty0 + 8 * b, (buse - 1) & 1, L.wait_ns)) &&
+                                           wait_phase(full0 + 8 * s, use & 1, L.wait_ns));
+          if (!ok) break;
+          tc_fence_after();
+          const uint64_t b0 = ring_desc + s * (kStageBytes >> 4);
+          const uint32_t d = tmem + b * kNT;
+          auto multiply = [&](int kb) {
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks)
+              mma_f8_ta(d, a_img + kb * 32 + ks * 8, b0 + kb * (kBlockBytes >> 4) + 2 * ks, idesc_u,
+                        (kb > 0 || ks > 0) ? 1u : 0u);
+          };
+          if (elect_one())
+            for (int kb = 0; kb + 1 < kblocks; ++kb) multiply(kb);
+          __syncwarp();
+          ok = __all_sync(0xFFFFFFFFu, wait_phase(tempty0 + 8 * (p % kBufs), (p / kBufs) & 1, L.wait_ns));
+          if (!ok) break;
+          tc_fence_after();
+          if (elect_one()) {
+            multiply(kblocks - 1);
+            mma_commit(empty0 + 8 * s);
+            mma_commit(tfull0 + 8 * b);
+          }
+          __syncwarp();
+          ++mmas;
+          ++cpass;
+          c = 1;
+        } else {
+          ok = __all_sync(0xFFFFFFFFu, wait_phase(aready, apass & 1, L.wait_ns));
+          if (!ok) break;
+          ++apass;
+          tc_fence_after();
         }
-        ++apass;
-        tc_fence_after();
         // sweep t - 1 is decided: its table's half takes the next step's
         if (tab_ahead && t + 1 < t_end) copy_table(t + 1);
-        for (int c = 0; c < nchunks && ok; ++c) {
+        for (; c < nchunks && ok; ++c) {
           const uint32_t b = cpass % kBufs, buse = cpass / kBufs;
           if (!__all_sync(0xFFFFFFFFu, buse == 0 || wait_phase(tempty0 + 8 * b, (buse - 1) & 1, L.wait_ns))) {
             ok = false;
@@ -312,7 +356,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
             tc_fence_after();
             if (elect_one()) {
               const uint64_t b0 = ring_desc + s * (kStageBytes >> 4);
-              const uint32_t a0 = tmem + kTmemA + kb0 * 32, d = tmem + b * kNT;
+              const uint32_t a0 = a_img + kb0 * 32, d = tmem + b * kNT;
 #pragma unroll
               for (int j = 0; j < kKPS; ++j)
                 if (j < nk) {
@@ -377,7 +421,8 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
 #pragma unroll
         for (int w = 0; w < kWordsPT; ++w)
           if (c < nchunks) {
-            put_spins32_tm(tlane, c * kNT + grp * kCols + 32 * w, cur[c][w], neg8);
+            put_spins32_tm(tlane + (two_images ? (t_begin & 1) * kImageCols : 0), c * kNT + grp * kCols + 32 * w,
+                           cur[c][w], neg8);
           }
       tmem_wait_st();
       tc_fence_before();
@@ -415,6 +460,19 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
         const uint32_t base = smem_u32(sTab) + half * kTabHalf * 4 + 4u * static_cast<uint32_t>(DIAG ? dk : imax);
         int* red = sRed + (t & 1) * kGroups * 128;
         int eacc = 0;
+        // Chunk c decided: with two images its new spins go into the next sweep's now; then TMEM
+        // buffer b, drained by this warp, is the MMA issuer's again.
+        const uint32_t next_img = tlane + ((t + 1) & 1) * kImageCols;
+        auto release = [&](int c, uint32_t b, uint32_t word) {
+          nxt[c][0] = word;
+          if (two_images && !last && warp_active) {
+            put_spins32_tm(next_img, c * kNT + grp * kCols, word, neg8);
+            tmem_wait_st();
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(tempty0 + 8 * b);
+        };
 #pragma unroll 1
         for (int c = 0; c < nchunks; ++c) {
           const uint32_t b = cpass % kBufs, buse = cpass / kBufs;
@@ -441,13 +499,9 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
               eacc += static_cast<int>(esum);
             }
           }
-          nxt[c][0] = word & valid_mask(c, 0);
-          // TMEM buffer b drained by this warp: let the MMA issuer reuse it.
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(tempty0 + 8 * b);
+          release(c, b, word & valid_mask(c, 0));
         }
-        if (!last && warp_active) {
+        if (!last && warp_active && !two_images) {
           // Every MMA of sweep t has completed (the last chunk's commit was awaited): the A
           // image can take s(t+1).
 #pragma unroll
@@ -469,7 +523,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
           }
           break;
         }
-        if (!last && etid == 0) mbar_arrive(aready);
+        if (!last && etid == 0 && !two_images) mbar_arrive(aready);
         int tot = 0;
 #pragma unroll
         for (int g = 0; g < kGroups; ++g) tot += red[g * 128 + row];
