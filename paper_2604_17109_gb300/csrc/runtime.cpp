@@ -2130,7 +2130,9 @@ int tune_slope(pim_instance* rep, int R, int flags, int force_nt, cudaStream_t s
   const int s_long = std::min(kTuneLong, steps), s_short = std::min(kTuneShort, s_long / 2);
   double best[2] = {1e30, 1e30};
   const int sweeps[2] = {s_short, s_long};
-  for (int pass = 0; pass < 2; ++pass)
+  // Over a few sweeps only, a microsecond's scatter of a launch would decide between variants.
+  const int passes = s_long - s_short >= 16 ? 2 : 8;
+  for (int pass = 0; pass < passes; ++pass)
     for (int v = 0; v < 2; ++v) {
       if (v == 0 && s_short < 1) continue;
       double ms = 0.0;
