@@ -89,8 +89,17 @@ FP4_BF16_NOMINAL = 13.5 / 2.25  # dense E2M1 / BF16 tensor rates (nominal, per G
 # workloads (dram__bytes_read.sum + dram__bytes_write.sum of one launch), as fixed + per-pass
 # bytes (passes = sweeps + 1).  They are recorded values, not measured by this script; a
 # workload whose kernel changed after its capture has no entry here (traffic reported null):
-# The kernels of sk200, sk4096 and maxcut8192 changed after their captures.
-DRAM_TRAFFIC: dict = {}
+#   sk200       sweep_tc_kernel<256,0,queue>, 100-sweep launch: 13.42 MB read + 0.04 MB
+#               written, of which one 2 KB threshold table per pass
+#   sk4096      sweep_big_kernel<64, E2M1 coupling-resident>, 50-sweep capture 10.22 MB = the
+#               8 MB E2M1 coupling image once + misc, and one 32 KB threshold table per pass
+#   maxcut8192  sweep_big_kernel<128,BF16>, 50-sweep capture 3.68 GB read + 0.22 GB written =
+#               what of the 134 MB image has left L2 when a pass comes back to it
+DRAM_TRAFFIC = {
+    "sk200": (13.42e6 + 0.036e6 - 101 * 2048.0, 2048.0),
+    "sk4096": (10.20e6 + 0.025e6 - 51 * 32768.0, 32768.0),
+    "maxcut8192": (0.0, (3.68e9 + 0.217e9) / 51),
+}
 
 
 def _schedule(sweeps: int):
