@@ -577,10 +577,10 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_big_kernel(const __grid_con
 #pragma unroll
                   for (int e = 0; e < 16; ++e) {
                     g[e] = __fadd_rn(tanh_approx(x[e]), ns[REAL ? 16 * c + e : 0]);
-                    least = fminf(least, fabsf(g[e]));
+                    least = min_nan(least, fabsf(g[e]));
                   }
                 }
-                if (__any_sync(0xFFFFFFFFu, least <= margin))
+                if (__any_sync(0xFFFFFFFFu, !(least > margin)))
                   settle_chunk<16>(g, x, static_cast<uint32_t>((col0 + 16 * c) >> 3), static_cast<uint32_t>(r),
                                    static_cast<uint32_t>(t), P.q, L.round_keys, cw16, margin, P.xi, eta, P.act,
                                    P.lut_levels, sZ);

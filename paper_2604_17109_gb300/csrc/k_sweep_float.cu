@@ -388,9 +388,9 @@ __global__ void __launch_bounds__(FloatCfg<CAP>::kBoundThreads, 1)
               for (int e = 0; e < W; ++e) {
                 x[e] = __fmul_rn(b, x[e]);
                 g[e] = __fadd_rn(tanh_approx(x[e]), g[e]);
-                least = fminf(least, fabsf(g[e]));
+                least = min_nan(least, fabsf(g[e]));
               }
-              if (__any_sync(0xFFFFFFFFu, least <= margin))
+              if (__any_sync(0xFFFFFFFFu, !(least > margin)))
                 settle_chunk<W>(g, x, c * W / 8, static_cast<uint32_t>(rg), static_cast<uint32_t>(t), q,
                                 L.round_keys, ob, margin, xi, eta, act, levels, sZ);
             }

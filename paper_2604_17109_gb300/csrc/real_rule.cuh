@@ -3,8 +3,8 @@
 //   x = b_t I, tau = tanh(x) (or the L-level staircase), delta = (tau + xi s) + eta_t z(key),
 //   s' = +1 iff delta >= 0.
 // The shortcut takes tanh from the hardware's approximation and the sign of its sum; where that
-// sum lies within a margin of zero, settle_chunk evaluates the rule itself, so every decision is
-// the rule's.
+// sum lies within a margin of zero or is NaN (an infinite b_t times a zero field), settle_chunk
+// evaluates the rule itself, so every decision is the rule's.  A NaN is no sum >= 0: the spin is -1.
 #pragma once
 #include <cmath>
 #include <cstdint>
@@ -28,8 +28,16 @@ __device__ __forceinline__ float tanh_approx(float x) {
   return y;
 }
 
-// The rule with tanh for the spins of a chunk (W spins from Philox block blk0 on) with |g| <= margin:
-// g = +1 or -1 from x = b I and the old spins ob.  Out of line: the common path keeps its registers.
+// The lesser of two values, NaN if either is (fminf would drop it).
+__device__ __forceinline__ float min_nan(float a, float b) {
+  float y;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+  return y;
+}
+
+// The rule with tanh for the spins of a chunk (W spins from Philox block blk0 on) that the shortcut
+// leaves open, |g| <= margin or NaN: g = +1 or -1 from x = b I and the old spins ob.  Out of line: the
+// common path keeps its registers.
 template <int W>
 __device__ __noinline__ void tanh_chunk(float* g, const float* x, uint32_t blk0, uint32_t r, uint32_t t,
                                         uint32_t q, const uint32_t* rk, uint32_t ob, float margin, float xi,
@@ -40,7 +48,7 @@ __device__ __noinline__ void tanh_chunk(float* g, const float* x, uint32_t blk0,
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       const int e = 8 * b + k;
-      if (fabsf(g[e]) <= margin) {
+      if (!(fabsf(g[e]) > margin)) {
         const float z = sZ[philox_half(o, k) >> 4];
         const float a = __fadd_rn(tanhf(x[e]), ((ob >> e) & 1u) ? xi : -xi);
         g[e] = __fadd_rn(a, __fmul_rn(eta, z)) >= 0.0f ? 1.0f : -1.0f;
@@ -67,8 +75,8 @@ __device__ __noinline__ void stairs_chunk(float* g, const float* x, uint32_t blk
   }
 }
 
-// Decides again the spins of a chunk that the shortcut leaves open (some lane has |g| <= margin;
-// with a staircase all of them).
+// Decides again the spins of a chunk that the shortcut leaves open (some lane has a g that is not
+// beyond the margin; with a staircase all of them).
 template <int W>
 __device__ __forceinline__ void settle_chunk(float (&g)[W], const float (&x)[W], uint32_t blk0, uint32_t r,
                                              uint32_t t, uint32_t q, const uint32_t* rk, uint32_t ob,
