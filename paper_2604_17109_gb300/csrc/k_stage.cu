@@ -185,6 +185,7 @@ cudaError_t launch_diag_thresholds(const uint32_t* d_thr, int steps, int imax, i
 // ---------------------------------------------------------------------------------------
 // Initial spin bits.  Philox mode: spin i of replica r is +1 iff bit 15 of its draw at
 // step field 0xFFFFFFFF is set.  Host mode: pack int8 +-1 (d_init[R][n], instance 0 only).
+// Bits past n are 0, in the best states too.
 // Grid: x = word, y = replica, z = problem.
 // ---------------------------------------------------------------------------------------
 __global__ void init_bits_kernel(const Problem* __restrict__ probs, const int8_t* __restrict__ init,
@@ -212,6 +213,8 @@ __global__ void init_bits_kernel(const Problem* __restrict__ probs, const int8_t
     }
   }
   P.cur_bits[static_cast<size_t>(r) * P.words + w] = bits;
+  // A sweep kernel may write its 16-spin chunks of the best states only; the rest of a row is 0.
+  if (w >= (P.n + 15) / 16 / 2) P.best_bits[static_cast<size_t>(r) * P.words + w] = 0;
 }
 
 cudaError_t launch_init_bits(const Problem* d_probs, int nprob, int maxR, int max_words,
