@@ -693,7 +693,7 @@ cudaError_t variant_setup(int smem, const void** fn, int* max_blocks) {
   if (e != cudaSuccess) return e;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  *max_blocks = per_sm * sms;
+  *max_blocks = resident_ctas(per_sm, BigCfg<NT, OP>::kTmemCols) * sms;
   return cudaSuccess;
 }
 

@@ -602,7 +602,7 @@ int sweep_mid_max_blocks() {
     return 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return per_sm * sms;
+  return resident_ctas(per_sm, kTmemCols) * sms;
 }
 
 int sweep_mid_table_words() { return kTabWords; }

@@ -1,5 +1,6 @@
 // Launch functions of the device kernels (host side, internal to the library).
 #pragma once
+#include <algorithm>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -18,6 +19,12 @@ __host__ __device__ inline uint32_t sw128_offset(int row, int k, int rows) {
   return static_cast<uint32_t>(kb) * rows * 128u + (row >> 3) * 1024u + (row & 7) * 128u +
          ((chunk ^ (row & 7)) << 4) + (k & 15);
 }
+
+// CTAs that one SM really holds at once: the occupancy call counts registers, threads and shared
+// memory but not tensor memory, of which an SM has 512 columns.  A kernel whose CTAs wait for one
+// another (the large-N kernel's grid barrier) must not be launched with more: a CTA past them would
+// wait in tcgen05.alloc for one that waits for it.
+inline int resident_ctas(int by_occupancy, int tmem_cols) { return std::min(by_occupancy, 512 / tmem_cols); }
 
 // Staging (once per instance).
 // diag != 0 puts that value on the diagonal of the image (inside n x n); e5m2 selects the
