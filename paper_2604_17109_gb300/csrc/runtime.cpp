@@ -497,10 +497,13 @@ void parallel_for(int count, F fn, int grain = 64, size_t work = SIZE_MAX) {
     return;
   }
   std::vector<std::thread> th;
+  th.reserve(nth);
   const int per = (count + nth - 1) / nth;
-  for (int k = 0; k < nth; ++k) {
-    const int b = k * per, e = std::min(count, b + per);
-    if (b < e) th.emplace_back(fn, b, e);
+  int b = 0;  // [0, b) is shared out
+  try {
+    for (; b < count; b = std::min(count, b + per)) th.emplace_back(fn, b, std::min(count, b + per));
+  } catch (const std::exception&) {
+    fn(b, count);  // no thread to be had: the rest runs here
   }
   for (auto& t : th) t.join();
 }
