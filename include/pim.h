@@ -268,7 +268,8 @@ void pim_batch_destroy(pim_batch* batch);
  * counterpart is the host-side task scheduling it replaces).  mode 0: the analytic cost model
  * only; mode 1 (default): pim_batch_create measures new shape classes first (see above).
  * When the environment variable PIM_TUNE_CACHE names a file, measured times are appended
- * to it and read back by later processes.
+ * to it and read back by later processes; times of another generation of the kernels are
+ * passed over.
  * Errors: PIM_ERR_INVALID (mode not 0 or 1).
  *
  * pim_tune_report -- the measured times, one line per shape class:

@@ -1291,6 +1291,9 @@ struct BigPlan {
 // NT) instance sweep.  The router and the large-N tile plan use a measured time wherever
 // the cache has one and the analytic model otherwise.  Entries are kept per process and,
 // when PIM_TUNE_CACHE names a file, appended to it and read back by later processes.
+// Lines of the file start with the generation of the kernels that were measured (raise it with a
+// kernel's speed): times of others, or of files from before it stood there, say nothing about these.
+constexpr char kTuneTag[] = "kernels2";
 std::mutex g_tune_mu;
 std::map<std::string, double> g_tune;  // key -> microseconds
 bool g_tune_loaded = false;
@@ -1330,9 +1333,10 @@ void tune_load_locked() {
   if (!f) return;
   char line[256];
   while (std::fgets(line, sizeof line, f)) {
-    char key[200];
+    char tag[16], key[200];
     double us = 0.0;
-    if (std::sscanf(line, "%199s %lf", key, &us) == 2 && us > 0.0) g_tune[key] = us;
+    if (std::sscanf(line, "%15s %199s %lf", tag, key, &us) == 3 && std::strcmp(tag, kTuneTag) == 0 && us > 0.0)
+      g_tune[key] = us;
   }
   std::fclose(f);
 }
@@ -1360,7 +1364,7 @@ void tune_store(const std::string& key, double us) {
   const char* path = std::getenv("PIM_TUNE_CACHE");
   if (path && *path) {
     if (FILE* f = std::fopen(path, "a")) {
-      std::fprintf(f, "%s %.6g\n", key.c_str(), us);
+      std::fprintf(f, "%s %s %.6g\n", kTuneTag, key.c_str(), us);
       std::fclose(f);
     }
   }
