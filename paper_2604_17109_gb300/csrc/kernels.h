@@ -22,7 +22,7 @@ __host__ __device__ inline uint32_t sw128_offset(int row, int k, int rows) {
 
 // CTAs that one SM really holds at once: the occupancy call counts registers, threads and shared
 // memory but not tensor memory, of which an SM has 512 columns.  A kernel whose CTAs wait for one
-// another (the large-N kernel's grid barrier) must not be launched with more: a CTA past them would
+// another (the large-N kernel's barriers) must not be launched with more: a CTA past them would
 // wait in tcgen05.alloc for one that waits for it.
 inline int resident_ctas(int by_occupancy, int tmem_cols) { return std::min(by_occupancy, 512 / tmem_cols); }
 

@@ -151,6 +151,8 @@ struct ServeQueue {
   uint64_t idle_ns;
 };
 
+constexpr int kBarWords = 32;  // a barrier counter of the large-N kernel has a 128-byte line of its own
+
 // Launch of the large-N kernel: one instance, all sweeps, cooperative grid of
 // (replica tiles) x (nt-spin column blocks).
 struct BigLaunch {
@@ -161,8 +163,8 @@ struct BigLaunch {
   float* energy;           // [3][rpad] rotating per-replica energy accumulators (zeroed);
                            // int32 for integer couplings, float for real couplings
   int nt;                  // output spins per CTA (64 or 128)
-  unsigned int* bar;       // grid barrier: 64-bit monotone arrival counter with an abort
-                           // bit (zeroed, 8-byte aligned)
+  unsigned int* bar;       // barriers, kBarWords apart, one per replica tile: 64-bit monotone
+                           // arrival counter with an abort bit (zeroed)
   int rbase;               // first replica of this launch
   int rpad;                // replica rows of this launch (multiple of 128)
   int ncb;                 // column blocks = npad / nt

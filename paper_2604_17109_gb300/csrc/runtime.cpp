@@ -1283,7 +1283,7 @@ struct BigPlan {
 // rate (about 64 GB/s per SM when all SMs stream, as measured for this kernel on GB300) and
 // its MMA time at the per-SM tensor rate (1889 TFLOP/s BF16, twice that for FP8, four times
 // for FP4, over 152 SMs); replica tiles that do not fit the co-resident grid run as further
-// launches, each with its own ~3 us grid barrier per sweep.
+// launches, each with its own ~3 us of barrier and bookkeeping per sweep.
 // ---- Autotuning: measured kernel times per shape class -----------------------------------
 // pim_batch_create (mode 1) times, on the batch's own instances, every shape class it has
 // not seen on this device before: the persistent mid-N kernel per (npad, decision path)
@@ -1416,6 +1416,9 @@ int plan_big(int n, int npad, int R, bool real, bool fp4, int stride_words, BigP
 // (two spin images, energy accumulators, barrier words) comes from the stream-ordered pool.
 // Bytes of one large-N spin image (bits) of rpad replica rows.
 size_t big_image_bytes(int rpad, int npad) { return static_cast<size_t>(rpad) * npad / 8; }
+// What a launch zeroes: energy accumulators and barrier words; and its whole scratch.
+size_t big_zeroed_bytes(int rpad) { return sizeof(float) * 3 * rpad + rpad / 128 * kBarWords * sizeof(uint32_t); }
+size_t big_scratch_bytes(int rpad, int npad) { return 2 * big_image_bytes(rpad, npad) + big_zeroed_bytes(rpad); }
 
 int launch_big(const Problem& P, bool real, int t_begin, int sweeps, uint64_t seed, bool cont,
                int* d_err, char* scratch, int* launches, cudaStream_t st) {
@@ -1430,12 +1433,10 @@ int launch_big(const Problem& P, bool real, int t_begin, int sweeps, uint64_t se
     const int tiles = std::min(plan.tiles_per_launch, tiles_total - tile0);
     const int rpad = tiles * 128;
     const size_t img_bytes = big_image_bytes(rpad, P.npad);
-    const size_t energy_bytes = sizeof(float) * 3 * rpad;
-    const size_t bytes = 2 * img_bytes + energy_bytes + 256;
     char* d = scratch;
     if (!scratch)
-      CK(run_alloc(reinterpret_cast<void**>(&d), bytes, st), "cudaMallocAsync large-N scratch");
-    CK(cudaMemsetAsync(d + 2 * img_bytes, 0, energy_bytes + 256, st), "clear large-N scratch");
+      CK(run_alloc(reinterpret_cast<void**>(&d), big_scratch_bytes(rpad, P.npad), st), "cudaMallocAsync large-N scratch");
+    CK(cudaMemsetAsync(d + 2 * img_bytes, 0, big_zeroed_bytes(rpad), st), "clear large-N scratch");
     BigLaunch L{};
     L.P = P;
     L.s_img[0] = reinterpret_cast<uint8_t*>(d);
@@ -1443,7 +1444,7 @@ int launch_big(const Problem& P, bool real, int t_begin, int sweeps, uint64_t se
     L.j4 = plan.op == kBigFp4 ? P.jimg4 : nullptr;
     L.tab_smem = smem.tab_smem;
     L.energy = reinterpret_cast<float*>(d + 2 * img_bytes);
-    L.bar = reinterpret_cast<unsigned int*>(d + 2 * img_bytes + energy_bytes);
+    L.bar = reinterpret_cast<unsigned int*>(d + 2 * img_bytes + sizeof(float) * 3 * rpad);
     L.nt = plan.nt;
     L.rbase = tile0 * 128;
     L.rpad = rpad;
@@ -1802,8 +1803,7 @@ int build_plan(pim_instance* const* insts, int count, const int* replicas, const
       const int rc = plan_big(P.n, P.npad, P.R, insts[k]->real, P.jimg4 != nullptr, P.stride_words, &plan);
       if (rc != PIM_OK) return rc;
       const int rpad = plan.tiles_per_launch * 128;
-      B.big_scratch = std::max(B.big_scratch, 2 * big_image_bytes(rpad, P.npad) +
-                                                  sizeof(float) * 3 * rpad + 256);
+      B.big_scratch = std::max(B.big_scratch, big_scratch_bytes(rpad, P.npad));
       continue;
     }
     const int g = group_of(k);
