@@ -568,7 +568,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_con
   }
 
   // ---- teardown: no copy or MMA of this CTA may still be in flight ------------------------
-  if (tid == 32) {
+  if (warp == 1 && elect_one()) {  // the lane that issued the MMAs: a commit covers its own thread's
     mma_commit(drain);
     wait_phase(drain, 0, L.wait_ns);
     for (uint32_t k = tabs_copied > 2 ? tabs_copied - 2 : 0; k < tabs_copied; ++k)
