@@ -6,13 +6,18 @@
 // pipe that runs integer multiply-adds, the shifts and logic fill the other integer pipe.  So what
 // can be is done in FP32 arithmetic, which both FP32 pipes run: an integer below 2^23 is the subnormal
 // float of the same bits, multiply-adds on those are exact, and subnormals run at full rate.  Against
-// integer arithmetic, us per sweep: SK N = 200, 100 instances x 1024 replicas 13.14 -> 12.85, Max-Cut
-// N = 100, 100 x 1024 7.19 -> 6.84, one SK N = 200 x 128 1.48 -> 1.36; with a bias N = 256, 200 x 256
-// 19.0 -> 13.4, N = 400, 80 x 256 30.2 -> 17.1.
+// integer arithmetic, us per sweep of runs of 100 (with a bias) to 1000 sweeps, launch included: SK
+// N = 200, 100 instances x 1024 replicas 13.14 -> 12.85 (12.3 over 2000 sweeps), Max-Cut N = 100, 100 x
+// 1024 7.19 -> 6.84, one SK N = 200 x 128 1.48 -> 1.36; with a bias N = 256, 200 x 256 19.0 -> 13.4,
+// N = 400, 80 x 256 30.2 -> 17.1 (16.7 with two spin images).
 #pragma once
 #include <cstdint>
 
 namespace pim {
+
+// An integer D, |D| < 2^22, held exactly in FP32 stands in the low mantissa bits of D + kMagic.
+constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23
+constexpr uint32_t kMagicBits = 0x4B400000u;
 
 // Shared-memory addresses of the 16-bit table entries of two exactly integral fields: base + 2 D.
 __device__ __forceinline__ void entry_address2(uint32_t d0, uint32_t d1, uint32_t base, uint32_t& a0,

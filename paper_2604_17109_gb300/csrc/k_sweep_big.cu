@@ -29,9 +29,10 @@
 //            the next sweep's K-loop every CTA reads the replica energies of s(t), updates best /
 //            first hit (redundantly, identically in all CTAs) and keeps its own spins of s(t)
 //            as the best state when the energy improved.
-// Measured (GB300, us per sweep; spins streamed as operand bytes before): BF16 N = 8192 x 256
-// replicas 40.1 -> 33.8, x 64 29.7 -> 26.2; BF16 N = 2000 x 256 11.3 -> 9.8, N = 1000 x 128 7.9 -> 6.9;
-// FP8 N = 4800 x 128 10.5 -> 10.0; E2M1 N = 4096 x 256 7.0 -> 6.7 (N = 1201 x 200 4.3 -> 4.6).
+// Measured (GB300, us per sweep; spins streamed as operand bytes before -> as bits -> with a barrier per
+// tile, runs of 40 to 100 sweeps): BF16 N = 8192 x 256 replicas 40.1 -> 33.8 -> 32.9, x 64 29.7 -> 26.2 ->
+// 26.7; BF16 N = 2000 x 256 11.3 -> 9.8 -> 9.2, N = 1000 x 128 7.9 -> 6.9 -> 6.6; FP8 N = 4800 x 128 10.5 ->
+// 10.0 -> 10.0; E2M1 N = 4096 x 256 7.0 -> 6.7 -> 6.6 (N = 1201 x 200 4.3 -> 4.6 -> 4.6).
 #include <algorithm>
 #include <cfloat>
 #include <climits>
@@ -46,13 +47,10 @@
 namespace pim {
 namespace {
 
-
 constexpr int kTabWords = 8192;     // threshold table of one step staged in shared memory
 constexpr int kEpiWarps = 16;
 constexpr int kThreads = (2 + kEpiWarps) * 32;
 constexpr int kSmemBudget = 227 * 1024;
-constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23: integer D (|D| < 2^22) in the low mantissa bits
-constexpr uint32_t kMagicBits = 0x4B400000u;
 
 // The K loop runs in stages of kPB K-blocks through a ring of kStages: the spins' operand in tensor
 // memory (32 columns, i.e. 128 bytes of every row, per K-block), expanded from the bit image by the

@@ -89,9 +89,6 @@ __device__ __forceinline__ void put_spins32_tm(uint32_t tlane, int col, uint32_t
                : "memory");
 }
 
-constexpr float kMagic = 12582912.0f;      // 1.5 * 2^23: integer D in the low mantissa bits
-constexpr uint32_t kMagicBits = 0x4B400000u;
-
 // A thread's 32 columns of one chunk (two 16-column halves): the TMEM load of each half runs while its
 // two Philox blocks are drawn (DECIDE: every sweep but the final energy pass), then the rule.  Returns
 // the new spins of the 32 columns as bits.
@@ -122,7 +119,7 @@ __device__ __forceinline__ uint32_t chunk32(uint32_t ta, uint32_t blk0, uint32_t
 }
 
 // The same columns with the table in global memory (imax >= 2048), or of a diagonal-encoded image
-// without its table.  Out of line: inlined, its sixteen table reads in flight spill the loop around it.  Returns the spins and the energy sum.
+// without its table, sixteen table reads in flight.  Returns the spins; the energy sum is added to eacc.
 __device__ __forceinline__ uint32_t table_chunk32(uint32_t ta, int col0, int n, const int* sH, int dg, uint32_t cw32,
                                                const uint16_t* tab16, bool last, uint32_t rg, uint32_t t,
                                                uint32_t q, const uint32_t* rk, int& eacc) {
@@ -159,8 +156,9 @@ __device__ __forceinline__ uint32_t table_chunk32(uint32_t ta, int col0, int n, 
 
 // One variant per MidMode keeps the register allocation of each to the path that it runs.  One kernel
 // for both general tables took 30.2 us per sweep at N = 400 with a bias (80 instances x 256 replicas)
-// and 23.7 at N = 700 with couplings of +-9 and a bias (60 x 256); these take 17.1 and 20.1, and a bias
-// unit beside one with a larger table, on the variant for global memory, 27.3.
+// and 23.7 at N = 700 with couplings of +-9 and a bias (60 x 256); these take 16.7 and 20.1 (runs of 100
+// sweeps; 15.6 and 19.2 a sweep without the launch), and the bias units of N = 400 beside one with a
+// larger table, on the variant for global memory, 24.7.
 template <int MODE>
 __global__ void __launch_bounds__(kThreads, 1) sweep_mid_kernel(const __grid_constant__ Launch L) {
   constexpr bool DIAG = MODE == kMidDiag;

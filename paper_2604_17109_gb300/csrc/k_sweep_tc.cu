@@ -18,9 +18,10 @@
 // Bound by issue slots and fixed latencies, not by the tensor pipe: 14.6 instructions per spin update,
 // two CTAs of 8 warps per SM so that one's MMAs and barrier overlap the other's decisions.  The MMAs are
 // issued by the elected lane of a converged warp (53 / 65 / 128 cycles per MMA at N = 64 / 128 / 256; a
-// lone lane in a divergent branch needs 84).  SK N = 200, 100 instances x 1024 replicas: 13.8 us per
-// sweep with that lone lane and integer arithmetic in the rule, 12.9 now (1.6e12 spin updates/s).
-// Slower: three column groups (14.3), the next chunk's noise drawn during the decisions (13.0 - 13.6).
+// lone lane in a divergent branch needs 84).  SK N = 200, 100 instances x 1024 replicas, us per sweep of
+// runs of 400 sweeps, launch included: 13.8 with that lone lane and integer arithmetic in the rule, 12.85
+// now (12.3 over 2000 sweeps, 1.66e12 spin updates/s).  Slower, in the same runs: three column groups
+// (14.3), the next chunk's noise drawn during the decisions (13.0 - 13.6).
 #include <climits>
 
 #include "int_rule.cuh"

@@ -1277,13 +1277,15 @@ struct BigPlan {
   double us_per_sweep = 0.0;  // model estimate
 };
 
-// Per-sweep time model of the large-N kernel.  Every CTA streams K-blocks of 128 x 128 B
-// spins (128 FP8, 64 BF16 or 256 E2M1 spins per row) plus, unless they are resident, nt x
-// 128 B of couplings; a K-block costs the larger of its ingest time at the per-SM bulk-copy
-// rate (about 64 GB/s per SM when all SMs stream, as measured for this kernel on GB300) and
-// its MMA time at the per-SM tensor rate (1889 TFLOP/s BF16, twice that for FP8, four times
-// for FP4, over 152 SMs); replica tiles that do not fit the co-resident grid run as further
-// launches, each with its own ~3 us of barrier and bookkeeping per sweep.
+// Per-sweep time model of the large-N kernel, for shapes that nothing was measured for.  It charges
+// every CTA K-blocks of 128 x 128 B spins (128 FP8, 64 BF16 or 256 E2M1 spins per row) plus, unless
+// they are resident, nt x 128 B of couplings; a K-block costs the larger of its ingest time at the
+// per-SM bulk-copy rate (about 64 GB/s per SM when all SMs stream) and its MMA time at the per-SM
+// tensor rate (1889 TFLOP/s BF16, twice that for FP8, four times for FP4, over 152 SMs); replica tiles
+// that do not fit the co-resident grid run as further launches, each with its own ~3 us of barrier and
+// bookkeeping per sweep.  The constants are those of the kernel that streamed spins as operand bytes.
+// Spins stream as bits now, so the model lies above the times (BF16 N = 8192 x 256: 68 us, 33 measured;
+// the mid-N unit below N = 512: 10 us, 6.9 measured) and serves to compare variants and kernels.
 // ---- Autotuning: measured kernel times per shape class -----------------------------------
 // pim_batch_create (mode 1) times, on the batch's own instances, every shape class it has
 // not seen on this device before: the persistent mid-N kernel per (npad, decision path)

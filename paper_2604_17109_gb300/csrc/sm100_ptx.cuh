@@ -347,17 +347,6 @@ __device__ __forceinline__ void tmem_wait_st() {
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
-// Eight spins (low 8 bits) -> eight packed E2M1 values, element k in nibble k (low nibble
-// first): +1 = 0x2, -1 = 0xA.  The spread moves bit k to bit 4k + 3 (the sign bit of
-// nibble k).
-__device__ __forceinline__ uint32_t e2m1x8_from_bits(uint32_t b) {
-  uint32_t x = b & 0xFFu;
-  x = (x | (x << 12)) & 0x000F000Fu;
-  x = (x | (x << 6)) & 0x03030303u;
-  x = (x | (x << 3)) & 0x11111111u;
-  return 0xAAAAAAAAu ^ (x << 3);
-}
-
 // D (+)= A B with A (128 x 32 FP8, K-major) in tensor memory at a_tmem.
 __device__ __forceinline__ void mma_f8_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc,
                                           uint32_t idesc, uint32_t accumulate) {
