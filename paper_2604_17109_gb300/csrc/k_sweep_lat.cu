@@ -16,9 +16,10 @@
 //    s(t+1) is multiplied) and one MMA warp, which also streams the threshold tables through a
 //    ring of four;
 //  - two accumulators, so a CTA never waits for a reader of the old fields.
-// Measured (GB300, us per sweep, one instance of 128 replicas: 4 CTAs of 32; k_sweep_tc.cu before):
-//   h = 0  n = 64  1.19 -> 0.87   n = 128  1.94 -> 1.13   n = 256  4.28 -> 1.73
-//   h != 0 n = 64  1.94 -> 0.85   n = 128  3.50 -> 1.25   n = 256  7.24 -> 2.03
+// Measured (GB300, us per sweep of 500-sweep runs, one instance of 128 replicas: 4 CTAs of 32;
+// k_sweep_tc.cu before):
+//   h = 0  n = 64  1.19 -> 0.78   n = 128  1.94 -> 1.12   n = 256  4.28 -> 1.65
+//   h != 0 n = 64  1.94 -> 0.81   n = 128  3.50 -> 1.24   n = 256  7.24 -> 1.93
 // What is left at n = 64 (cycles of 1650): MMA with its barriers 870, lookups 320, write-back 370.
 // Measured slower: waits that spin without suspending (+8 %), the bookkeeping wait ahead of the
 // noise (+18 %), the MMAs issued by a decision warp after a named barrier (+11 %).
